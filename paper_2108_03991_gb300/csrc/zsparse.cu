@@ -9,16 +9,18 @@
 // solver; here the kept pattern of each object is reordered by reverse Cuthill-McKee (host), so
 // that L_s becomes a band of half-width b, factorised without pivoting in FP64 (one CTA per
 // object), and each product is the sparse rows of K_s + I_x/2 (all objects in one launch) and
-// then one warp per object for a forward and a back substitution, blocked by kZspBW columns
-// (each column of L and of U stored contiguously, a block's columns streamed into shared memory
-// by one bulk copy while the warp works on the previous block). C = Y_eq Z stays dense, so j = h - C h is unchanged and e = Z_s h, needed only by the
-// I_x e term of the system matvec, runs beside it. The sparse form is used when every object
+// then one CTA per object for a forward and a back substitution, blocked by W columns (each
+// column of L and of U stored contiguously, the triangle of a diagonal block replaced by its
+// inverse, a block's columns streamed into shared memory by one bulk copy while earlier blocks
+// are worked on). C = Y_eq Z stays dense, so j = h - C h is unchanged and e = Z_s h, needed only
+// by the I_x e term of the system matvec, runs beside it. The sparse form is used when every object
 // qualifies (band and rows below half the dense bytes, b <= 256) and a set-up check of Z_s h
 // against the dense Z h (FP64, one probe vector) stays below 1e-8.
 #include <algorithm>
 #include <cmath>
 #include <complex>
 #include <memory>
+#include <type_traits>
 #include <vector>
 
 #include "bulk.cuh"
@@ -28,12 +30,15 @@ namespace bem {
 
 constexpr double kZspCut = 23.0;     // R_cut / delta
 constexpr int kZspBandMax = 192;     // largest half-bandwidth of the product kernel
-constexpr size_t kZspSmemMax = 220 * 1024;  // its shared memory (FP64: vector and two slabs)
-constexpr int kZspRows = (kZspBandMax + 31) / 32;  // rows per lane in a block's update
-// columns per block of the substitutions (slab: kZspBW b entries). 8: a warp's shared memory
-// (the vector and two slabs) is 22 KB at b = 114, so all the objects' warps are resident at once;
-// 16 and 32 took 30% and 70% longer per product on the 32 x 32 ring array
-constexpr int kZspBW = 8;
+constexpr size_t kZspSmemMax = 220 * 1024;  // FP64 vector and two 8-column slabs (set-up limit)
+constexpr size_t kZspSmemCta = 227 * 1024;  // shared memory of one CTA
+constexpr int kZspThreads = 256;  // consumers; one more warp issues the copies
+// columns per block of the substitutions: a step solves one block and updates the b rows beside
+// it. 32 in FP32; 16 in FP64, where a step is bound by the FP64 rate and wider slabs only take
+// shared memory (8 where the vector leaves no room for two 16-column slabs)
+constexpr int kZspW32 = 32, kZspW64 = 16, kZspW64s = 8;
+constexpr int kZspRing = 256;        // second accumulator, a ring over rows (>= 192 + 32)
+constexpr int kZspStages = 3;        // slabs in flight (2 where shared memory leaves no room)
 constexpr double kZspCheck = 1e-8;   // set-up check of Z_s h against Z h
 constexpr double kTwoPi = 6.283185307179586476925;
 
@@ -50,7 +55,8 @@ struct Zsp {
   int32_t *d_perm = nullptr, *d_pos = nullptr;  // row e0 + r <-> edge e0 + perm[r], both global
   int32_t *d_row = nullptr, *d_col = nullptr;   // K_s + I_x/2 in permuted row order (CSR)
   int64_t nnz = 0, nband = 0, nwork = 0;
-  int bmax = 0, nmax = 0;
+  int bmax = 0, bstore = 0, nmax = 0;  // largest half-bandwidth, largest stored one (>= 31)
+  int w64 = kZspW64;                   // columns per block of the FP64 substitutions
   double2* W = nullptr;                          // FP64 bands during set-up
   double2 *kv64 = nullptr, *L64 = nullptr, *U64 = nullptr, *D64 = nullptr;
   float2 *kv32 = nullptr, *L32 = nullptr, *U32 = nullptr, *D32 = nullptr;
@@ -165,6 +171,12 @@ __global__ void __launch_bounds__(256) k_zsp_lu(const ZspObj* objs, double2* Wal
   }
 }
 
+template <typename V> __device__ __forceinline__ V to_v(double2 a);
+template <> __device__ __forceinline__ double2 to_v<double2>(double2 a) { return a; }
+template <> __device__ __forceinline__ float2 to_v<float2>(double2 a) {
+  return make_float2((float)a.x, (float)a.y);
+}
+
 // column tables for the substitutions: Lc[c][k] = L[c+1+k][c], Uc[c][k] = U[c-1-k][c] (zero
 // outside the matrix), D[c] = 1 / U[c][c]; FP64 and FP32 copies
 __global__ void k_zsp_extract(const ZspObj* objs, const double2* Wall, double2* L64, double2* U64,
@@ -191,6 +203,50 @@ __global__ void k_zsp_extract(const ZspObj* objs, const double2* Wall, double2* 
   }
 }
 
+// Inverses of the triangles inside the W-column diagonal blocks, in place of the triangles: the
+// strict lower part of (L_ss)^-1 and the strict upper part of (U_ss)^-1 have as many entries as
+// the triangles themselves, so the column tables keep their size and layout (the half-bandwidth
+// stored is at least W - 1, so that a block's whole triangle lies in the band). A block's solve is
+// then a product, not a chain of W dependent steps. From the FP64 factors; one CTA of 32 threads
+// per block, one thread per column.
+template <int W, typename V>
+__global__ void __launch_bounds__(32) k_zsp_invtri(const ZspObj* objs, const double2* Wall, V* Lc,
+                                                   V* Uc) {
+  const ZspObj o = objs[blockIdx.y];
+  const int n = o.n, b = o.b, w = 2 * b + 1, c0 = W * blockIdx.x;
+  if (c0 >= n) return;
+  const int nb = min(W, n - c0), t = threadIdx.x;
+  const double2* A = Wall + o.woff;
+  __shared__ double2 T[W][W + 1], X[W][W + 1];
+  for (int i = t; i < nb * nb; i += 32) {
+    const int r = i / nb, q = i % nb;
+    T[r][q] = A[(int64_t)(c0 + r) * w + (q - r + b)];
+  }
+  __syncwarp();
+  if (t < nb) {  // column t of the unit lower inverse
+    X[t][t] = make_double2(1.0, 0.0);
+    for (int r = t + 1; r < nb; ++r) {
+      double2 acc = make_double2(0.0, 0.0);
+      for (int q = t; q < r; ++q) cfma(acc, T[r][q], X[q][t]);
+      X[r][t] = make_double2(-acc.x, -acc.y);
+      Lc[o.loff + (int64_t)(c0 + t) * b + (r - t - 1)] = to_v<V>(X[r][t]);
+    }
+    // column t of the upper inverse
+    auto inv = [](double2 d) {
+      const double den = d.x * d.x + d.y * d.y;
+      return make_double2(d.x / den, -d.y / den);
+    };
+    X[t][t] = inv(T[t][t]);
+    for (int r = t - 1; r >= 0; --r) {
+      double2 acc = make_double2(0.0, 0.0);
+      for (int q = r + 1; q <= t; ++q) cfma(acc, T[r][q], X[q][t]);
+      const double2 v = cmul(acc, inv(T[r][r]));
+      X[r][t] = make_double2(-v.x, -v.y);
+      Uc[o.loff + (int64_t)(c0 + t) * b + (t - r - 1)] = to_v<V>(X[r][t]);
+    }
+  }
+}
+
 __global__ void k_round_kv(const double2* a, float2* b, int64_t n) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) b[i] = make_float2((float)a[i].x, (float)a[i].y);
@@ -198,29 +254,19 @@ __global__ void k_round_kv(const double2* a, float2* b, int64_t n) {
 
 // ---------------------------------------------------------------------------------------
 // the product e = Z_s h in two launches: the rows of K_s + I_x/2 (all objects' rows in one
-// launch, eight lanes per row), then the substitutions (one warp per object and right-hand
-// side), blocked by kZspBW columns: the warp solves a block's triangle in registers (shuffles,
-// the triangle's entries read up front) and then applies the block's solved values to the b
-// rows below (above, going back) it as a small dense product, every lane on several rows at
-// once, instead of walking the band one column at a time.
+// launch, kZspLanes lanes per row), then the substitutions, one CTA per object and right-hand side,
+// blocked by W columns: a block is solved as a product with its stored triangle inverse and its
+// solved values are applied to the b rows below (above, going back).
 // ---------------------------------------------------------------------------------------
 template <typename V> __device__ __forceinline__ V vzero() { V v; v.x = 0; v.y = 0; return v; }
+template <typename V> __device__ __forceinline__ V one() { V v; v.x = 1; v.y = 0; return v; }
 template <typename V> __device__ __forceinline__ V vmul(V a, V b) {
   V r;
   r.x = a.x * b.x - a.y * b.y;
   r.y = a.x * b.y + a.y * b.x;
   return r;
 }
-template <typename V> __device__ __forceinline__ void vfma(V a, V b, V& acc) {
-  acc.x += a.x * b.x - a.y * b.y;
-  acc.y += a.x * b.y + a.y * b.x;
-}
-template <typename V> __device__ __forceinline__ V vshfl(V a, int src) {
-  V r;
-  r.x = __shfl_sync(0xffffffffu, a.x, src);
-  r.y = __shfl_sync(0xffffffffu, a.y, src);
-  return r;
-}
+constexpr int kZspLanes = 16;  // lanes per row of K_s + I_x/2: four entries each in flight
 
 // v[r] (permuted row r of every object, stride vs per right-hand side) = ((K_s + I_x/2) h)[perm r]
 template <typename R>
@@ -231,165 +277,183 @@ __global__ void __launch_bounds__(256) k_zsp_rows(const int32_t* __restrict__ ro
                                                   typename C2<R>::T* __restrict__ v, int64_t vs,
                                                   int ne) {
   typedef typename C2<R>::T V;
-  const int r = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 3);
-  const int sub = threadIdx.x & 7;
+  const int r = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kZspLanes);
+  const int sub = threadIdx.x & (kZspLanes - 1);
   const V* h = x + blockIdx.y * xs;
   V acc = vzero<V>();
-  if (r < ne)
-    for (int k = row[r] + sub; k < row[r + 1]; k += 8) vfma(kv[k], h[col[k]], acc);
+  if (r < ne) {
+    const int k1 = row[r + 1];
+    for (int k = row[r] + sub; k < k1; k += 4 * kZspLanes) {
+      // the missing entries of a short last group repeat its first column, with value 0
+      int c[4];
+      V a[4];
 #pragma unroll
-  for (int o = 4; o > 0; o >>= 1) {
+      for (int q = 0; q < 4; ++q) {
+        const int kk = k + q * kZspLanes;
+        c[q] = col[kk < k1 ? kk : k];
+        a[q] = kk < k1 ? kv[kk] : vzero<V>();
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cfma(acc, a[q], h[c[q]]);
+    }
+  }
+#pragma unroll
+  for (int o = kZspLanes / 2; o > 0; o >>= 1) {
     acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
     acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
   }
   if (r < ne && sub == 0) v[blockIdx.y * vs + r] = acc;
 }
 
-// one warp per (object, right-hand side): the band's slabs of kZspBW columns (of L forward, of U
-// going back) are streamed into two shared-memory slots by bulk copies, the next slab in flight
-// while the warp works on the current one; every wait is bounded and a timeout sets *err
-template <typename R>
-__global__ void __launch_bounds__(32) k_zsp_solve(const ZspObj* __restrict__ objs,
-                                                  const int32_t* __restrict__ perm,
-                                                  const typename C2<R>::T* __restrict__ Lc,
-                                                  const typename C2<R>::T* __restrict__ Uc,
-                                                  const typename C2<R>::T* __restrict__ D,
-                                                  const typename C2<R>::T* __restrict__ vin,
-                                                  int64_t vs, typename C2<R>::T* __restrict__ y,
-                                                  int64_t ys, int vbytes, int slab_bytes, int* err) {
+// One CTA per (right-hand side, object). The serial chain is 2 n / W block steps; a step is two
+// products out of shared memory with a barrier after each:
+//   solve   x_s = T_s^-1 r_s, eight lanes per row
+//   update  r -= (the W columns of the band beside the block) x_s, one lane per row, the columns
+//           split between the two halves of the CTA; the halves add into two accumulators (the
+//           vector, and a ring of kZspRing rows that covers the band), so they need no reduction
+// The slabs of W columns (contiguous, W b entries) arrive by bulk copies kept nst - 1 blocks
+// ahead. FP32: bound by moving a ring's 1.7 MB of tables through one SM (13 us at 64 B a clock)
+// when rings are few and by HBM when they fill the GPU; FP64 by the FP64 rate (0.2 ms a ring).
+// One warp per ring and 8-column blocks solved by shuffles, the form before, was one chain of
+// 2 n / 8 steps: e = Z_s h of rings of 912 edges (b = 114), k_zsp_rows included, took 297 us for
+// 1 ring, 306 for 36, 380 for 256 (FP64 2,810, 2,895, 3,187 us); now 57, 64, 125 us (FP64 408, 453,
+// 979). 2 to 7 slabs in flight take the same time.
+// Every wait is bounded; a timeout sets *err and ends the CTA once its copies have landed.
+template <typename R, int W>
+__global__ void __launch_bounds__(kZspThreads + 32) k_zsp_solve(
+    const ZspObj* __restrict__ objs, const int32_t* __restrict__ perm,
+    const typename C2<R>::T* __restrict__ Lc, const typename C2<R>::T* __restrict__ Uc,
+    const typename C2<R>::T* __restrict__ D, const typename C2<R>::T* __restrict__ vin, int64_t vs,
+    typename C2<R>::T* __restrict__ y, int64_t ys, int vbytes, int slab_bytes, int nst, int* err) {
   typedef typename C2<R>::T V;
   extern __shared__ __align__(16) unsigned char zsp_smem[];
-  uint64_t* bar = reinterpret_cast<uint64_t*>(zsp_smem);
-  V* v = reinterpret_cast<V*>(zsp_smem + 16);
-  unsigned char* slabs = zsp_smem + 16 + vbytes;  // two slots of slab_bytes
-  const ZspObj o = objs[blockIdx.x];
-  const int l = threadIdx.x;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(zsp_smem);  // [nst], nst <= 8
+  V* xs = reinterpret_cast<V*>(zsp_smem + 64);            // the block's solved values [W]
+  V* v1 = xs + W;                                         // second accumulator [kZspRing]
+  V* v = v1 + kZspRing;                                   // the running vector
+  unsigned char* slabs = reinterpret_cast<unsigned char*>(v) + vbytes;  // nst slots of slab_bytes
+  const ZspObj o = objs[blockIdx.y];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n = o.n, b = o.b, e0 = o.e0;
   const V* Lo = Lc + o.loff;
   const V* Uo = Uc + o.loff;
-  const int nblk = (n + kZspBW - 1) / kZspBW, nslab = 2 * nblk;
+  const int nblk = (n + W - 1) / W, nslab = 2 * nblk;
   // slab s: L's columns of block s (forward), then U's of block 2 nblk - 1 - s (going back)
-  auto issue = [&](int s) {
-    if (l == 0 && s < nslab) {
-      const int kb = s < nblk ? s : nslab - 1 - s;
-      const int c0 = kZspBW * kb, nb = min(kZspBW, n - c0);
-      const uint32_t bytes = (uint32_t)(((size_t)nb * b * sizeof(V) + 15) & ~(size_t)15);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // earlier reads of the slot
-      mbar_arrive_tx(&bar[s & 1], bytes);
-      bulk_g2s(slabs + (s & 1) * slab_bytes, (s < nblk ? Lo : Uo) + (int64_t)c0 * b, bytes, &bar[s & 1]);
-    }
+  auto issue = [&](int s, int slot) {
+    const int kb = s < nblk ? s : nslab - 1 - s;
+    const int c0 = W * kb, nb = min(W, n - c0);
+    const uint32_t bytes = (uint32_t)(((size_t)nb * b * sizeof(V) + 15) & ~(size_t)15);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // earlier reads of the slot
+    mbar_arrive_tx(&bar[slot], bytes);
+    bulk_g2s(slabs + (size_t)slot * slab_bytes, (s < nblk ? Lo : Uo) + (int64_t)c0 * b, bytes, &bar[slot]);
   };
-  if (l == 0) {
-    mbar_init(&bar[0], 1);
-    mbar_init(&bar[1], 1);
+  const bool producer = tid == kZspThreads;
+  if (producer) {
+    for (int q = 0; q < nst; ++q) mbar_init(&bar[q], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int q = 0; q < nst && q < nslab; ++q) issue(q, q);
   }
-  __syncwarp();
-  issue(0);
-  const V* vi = vin + blockIdx.y * vs + e0;
-  V* e = y + blockIdx.y * ys;
-  for (int r = l; r < n; r += 32) v[r] = vi[r];
-  __syncwarp();
+  const V* vi = vin + blockIdx.x * vs + e0;
+  for (int r = tid; r < n; r += kZspThreads + 32) v[r] = vi[r];
+  for (int r = tid; r < kZspRing; r += kZspThreads + 32) v1[r] = vzero<V>();
+  __syncthreads();
+  if (warp == kZspThreads / 32) {  // the copies: their issue stays off the consumers' chain
+    for (int s = 0; s < nslab; ++s) {
+      if (__syncthreads_or(0)) return;
+      __syncthreads();
+      if (producer && s + nst < nslab) issue(s + nst, s % nst);
+    }
+    return;
+  }
+  const int row = tid >> 3, sub = tid & 7;          // solve: row of the block, lane of the row
+  const int half = warp >> 2, i0 = (warp & 3) * 32 + lane;  // update: column half, row
+  int slot = 0, phase = 0;
+  V dn = vzero<V>();  // 1 / U_rr of this thread's row in the next block (read one step ahead)
+  auto step = [&](int s, auto dir) -> bool {
+    constexpr bool kFwd = decltype(dir)::value;
+    const bool ok = mbar_wait(&bar[slot], phase);
+    const V* S = reinterpret_cast<const V*>(slabs + (size_t)slot * slab_bytes);  // S[t b + k]: column t, entry k
+    const int c0 = W * (kFwd ? s : nslab - 1 - s), nb = min(W, n - c0);
+    const V dr = dn;
+    if (s + 1 >= nblk && s + 1 < nslab) dn = D[e0 + min(n - 1, W * (nslab - 2 - s) + row)];
+    // loads are unconditional (their addresses stay inside this CTA's shared memory) and what
+    // does not belong is dropped afterwards, so that a thread's loads are all in flight at once
+    V acc = vzero<V>();
+    if (row < W) {
+#pragma unroll
+      for (int q = 0; q < W / 8; ++q) {
+        const int t = sub + 8 * q;
+        V r = v[c0 + t];
+        const V r1 = v1[(c0 + t) & (kZspRing - 1)];
+        r.x += r1.x;
+        r.y += r1.y;
+        const int k = kFwd ? row - t - 1 : t - row - 1;
+        V a = S[t * b + max(k, 0)];
+        if (t == row) a = kFwd ? one<V>() : dr;
+        if (k >= -1 && t < nb && row < nb) cfma(acc, a, r);
+      }
+    }
+#pragma unroll
+    for (int q = 4; q > 0; q >>= 1) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, q);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, q);
+    }
+    if (sub == 0 && row < W) xs[row] = acc;
+    if (__syncthreads_or(!ok)) {
+      if (tid == 0) {
+        atomicExch(err, 1);
+        for (int q = 1; q < nst && s + q < nslab; ++q) {  // the copies in flight
+          const int sl = (slot + q) % nst;
+          mbar_wait(&bar[sl], sl > slot ? phase : phase ^ 1);
+        }
+      }
+      return false;
+    }
+    const int live = min(b, kFwd ? n - c0 - W : c0);  // rows beside the block (none below a short one)
+    for (int i = i0; i < live; i += 128) {
+      // entry k = W - 1 + i - t below the block, t + i above it; k < b belongs to column t
+      const int st = kFwd ? b - 1 : b + 1;
+      const V* p = S + half * (W / 2) * st + (kFwd ? W - 1 + i : i);
+      const int tlo = W + i - b - half * (W / 2), thi = min(nb, b - i) - half * (W / 2);
+      const V* x = xs + half * (W / 2);
+      V c[2] = {vzero<V>(), vzero<V>()};
+#pragma unroll
+      for (int q = 0; q < W / 2; ++q) {
+        const V a = p[q * st];
+        if (kFwd ? q >= tlo : q < thi) cfma(c[q & 1], a, x[q]);
+      }
+      const int g = kFwd ? c0 + W + i : c0 - 1 - i;
+      V* u = half ? &v1[g & (kZspRing - 1)] : &v[g];
+      u->x -= c[0].x + c[1].x;
+      u->y -= c[0].y + c[1].y;
+    }
+    if (tid < nb) {
+      const V x = xs[tid];
+      v1[(c0 + tid) & (kZspRing - 1)] = vzero<V>();
+      v[c0 + tid] = x;
+    }
+    __syncthreads();
+    if (++slot == nst) {
+      slot = 0;
+      phase ^= 1;
+    }
+    return true;
+  };
+  for (int s = 0; s < nblk; ++s)
+    if (!step(s, std::true_type())) return;
+  for (int s = nblk; s < nslab; ++s)
+    if (!step(s, std::false_type())) return;
   V al;
   al.x = (R)o.ar;
   al.y = (R)o.ai;
-  for (int s = 0; s < nslab; ++s) {
-    issue(s + 1);
-    if (!mbar_wait(&bar[s & 1], (s >> 1) & 1)) {
-      if (l == 0) atomicExch(err, 1);
-      if (s + 1 < nslab) mbar_wait(&bar[(s + 1) & 1], ((s + 1) >> 1) & 1);  // the copy in flight
-      return;
-    }
-    const V* S = reinterpret_cast<const V*>(slabs + (s & 1) * slab_bytes);  // S[t b + k]: column c0 + t, entry k
-    if (s < nblk) {
-      // forward substitution with the unit lower band, block s
-      const int c0 = kZspBW * s, nb = min(kZspBW, n - c0);
-      V tri[kZspBW - 1];
-#pragma unroll
-      for (int t = 0; t < kZspBW - 1; ++t) {  // L[c0+l][c0+t] for t < l
-        const int k = l - t - 1;
-        tri[t] = (k >= 0 && k < b && l < nb) ? S[t * b + k] : vzero<V>();
-      }
-      V yl = l < nb ? v[c0 + l] : vzero<V>();
-#pragma unroll
-      for (int t = 0; t < kZspBW - 1; ++t) {
-        if (t < nb) {
-          const V u = vmul(tri[t], vshfl(yl, t));
-          yl.x -= u.x;
-          yl.y -= u.y;
-        }
-      }
-      if (l < nb) v[c0 + l] = yl;
-      // the block's solved values on the b rows below it: lane l takes rows c0 + nb + l + 32 r,
-      // all of them at once (independent sums, each x_t broadcast once)
-      const int rend = min(n, c0 + nb + b);
-      V acc[kZspRows];
-#pragma unroll
-      for (int r = 0; r < kZspRows; ++r) acc[r] = vzero<V>();
-      for (int t = 0; t < nb; ++t) {
-        const V xt = vshfl(yl, t);
-#pragma unroll
-        for (int r = 0; r < kZspRows; ++r) {
-          const int i = c0 + nb + l + 32 * r, k = nb + l + 32 * r - t - 1;
-          if (i < rend && k < b) vfma(S[t * b + k], xt, acc[r]);
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < kZspRows; ++r) {
-        const int i = c0 + nb + l + 32 * r;
-        if (i < rend) {
-          v[i].x -= acc[r].x;
-          v[i].y -= acc[r].y;
-        }
-      }
-    } else {
-      // back substitution with U, block 2 nblk - 1 - s; x goes out as e = alpha x (unpermuted)
-      const int c0 = kZspBW * (nslab - 1 - s), nb = min(kZspBW, n - c0);
-      V tri[kZspBW];
-#pragma unroll
-      for (int t = 0; t < kZspBW; ++t) {  // U[c0+l][c0+t] for t > l
-        const int k = t - l - 1;
-        tri[t] = (k >= 0 && k < b && t < nb) ? S[t * b + k] : vzero<V>();
-      }
-      const V dl = l < nb ? D[e0 + c0 + l] : vzero<V>();
-      V yl = l < nb ? v[c0 + l] : vzero<V>();
-#pragma unroll
-      for (int t = kZspBW - 1; t >= 0; --t) {
-        if (t < nb) {
-          const V w = vmul(tri[t], vshfl(vmul(yl, dl), t));  // x_t = y_t / U_tt, final here
-          yl.x -= w.x;
-          yl.y -= w.y;
-        }
-      }
-      const V xl = vmul(yl, dl);
-      if (l < nb) {
-        v[c0 + l] = xl;
-        e[perm[e0 + c0 + l]] = vmul(al, xl);
-      }
-      // on the b rows above the block: lane l takes rows c0 - 1 - l - 32 r
-      const int rlo = max(0, c0 - b);
-      V acc[kZspRows];
-#pragma unroll
-      for (int r = 0; r < kZspRows; ++r) acc[r] = vzero<V>();
-      for (int t = 0; t < nb; ++t) {
-        const V xt = vshfl(xl, t);
-#pragma unroll
-        for (int r = 0; r < kZspRows; ++r) {
-          const int i = c0 - 1 - l - 32 * r, k = t + l + 32 * r;
-          if (i >= rlo && k < b) vfma(S[t * b + k], xt, acc[r]);
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < kZspRows; ++r) {
-        const int i = c0 - 1 - l - 32 * r;
-        if (i >= rlo) {
-          v[i].x -= acc[r].x;
-          v[i].y -= acc[r].y;
-        }
-      }
-    }
-    __syncwarp();
-  }
+  V* e = y + blockIdx.x * ys;
+  for (int r = tid; r < n; r += kZspThreads) e[perm[e0 + r]] = vmul(al, v[r]);
+}
+
+// shared memory of k_zsp_solve with nst slabs of w columns
+template <typename V> static size_t zsp_smem_bytes(const Zsp* z, int w, int nst) {
+  const size_t vbytes = ((size_t)z->nmax * sizeof(V) + 15) & ~(size_t)15;
+  return 64 + (size_t)(w + kZspRing) * sizeof(V) + vbytes + ((size_t)nst * w * z->bstore + w) * sizeof(V);  // + w: reads past the last slab, dropped
 }
 
 template <typename R>
@@ -408,20 +472,26 @@ int zsp_apply(aim_ctx* c, const typename C2<R>::T* h, typename C2<R>::T* e, int 
   const bool f = sizeof(R) == 4;
   V* v = f ? (V*)z->v32 : (V*)z->v64;
   const int ne = c->ne;
-  k_zsp_rows<R><<<dim3((unsigned)(((int64_t)ne * 8 + 255) / 256), nrhs), 256, 0, s>>>(
+  k_zsp_rows<R><<<dim3((unsigned)(((int64_t)ne * kZspLanes + 255) / 256), nrhs), 256, 0, s>>>(
       z->d_row, z->d_col, f ? (const V*)z->kv32 : (const V*)z->kv64, h, hs, v, ne, ne);
+  const int w = f ? kZspW32 : z->w64;
+  const int nst = zsp_smem_bytes<V>(z, w, kZspStages) <= kZspSmemCta ? kZspStages : 2;
+  const size_t sm = zsp_smem_bytes<V>(z, w, nst);
   const int vbytes = (int)(((size_t)z->nmax * sizeof(V) + 15) & ~(size_t)15);
-  const int slab_bytes = kZspBW * z->bmax * (int)sizeof(V);
-  const size_t sm = 16 + (size_t)vbytes + 2 * (size_t)slab_bytes;
-  static size_t attr = 48 * 1024;  // dynamic shared memory allowed so far
-  if (sm > attr) {
-    BEM_CUDA(cudaFuncSetAttribute(k_zsp_solve<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    attr = sm;
-  }
-  k_zsp_solve<R><<<dim3((unsigned)z->obj.size(), nrhs), 32, sm, s>>>(
-      z->d_obj, z->d_perm, f ? (const V*)z->L32 : (const V*)z->L64,
-      f ? (const V*)z->U32 : (const V*)z->U64, f ? (const V*)z->D32 : (const V*)z->D64, v, ne, e,
-      es, vbytes, slab_bytes, z->d_err);
+  const int slab_bytes = w * z->bstore * (int)sizeof(V);
+  auto launch = [&](auto* kernel) -> int {
+    // per call: the attribute belongs to the current device
+    BEM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    // the right-hand sides of one object next to each other: they share its tables in L2
+    kernel<<<dim3(nrhs, (unsigned)z->obj.size()), kZspThreads + 32, sm, s>>>(
+        z->d_obj, z->d_perm, f ? (const V*)z->L32 : (const V*)z->L64,
+        f ? (const V*)z->U32 : (const V*)z->U64, f ? (const V*)z->D32 : (const V*)z->D64, v, ne, e,
+        es, vbytes, slab_bytes, nst, z->d_err);
+    return BEM_OK;
+  };
+  if constexpr (sizeof(R) == 4) BEM_TRY(launch(&k_zsp_solve<R, kZspW32>));
+  else if (z->w64 == kZspW64) BEM_TRY(launch(&k_zsp_solve<R, kZspW64>));
+  else BEM_TRY(launch(&k_zsp_solve<R, kZspW64s>));
   BEM_CUDA(cudaGetLastError());
   return BEM_OK;
 }
@@ -515,7 +585,7 @@ int zsp_prepare(aim_ctx* c, const double* d_verts, const int32_t* d_tris, const 
   std::vector<int32_t> perm(c->ne), pos(c->ne), row(c->ne + 1, 0), col;
   std::vector<uint8_t> mask(nmax * nmax);
   std::vector<int> rp, ci;
-  int64_t nband = 0, nwork = 0;
+  int64_t nband = 0, nband_true = 0, nwork = 0;
   for (int i = 0; i < nobj; ++i) {
     const int e0 = c->e0[i], n = c->e1[i] - e0;
     k_zsp_mask<<<(unsigned)(((int64_t)n * n + 255) / 256), 256>>>(d_cen, rad, c->d_et, e0, n,
@@ -537,6 +607,9 @@ int zsp_prepare(aim_ctx* c, const double* d_verts, const int32_t* d_tris, const 
       for (int k = rp[m]; k < rp[m + 1]; ++k) b = std::max(b, std::abs(p[m] - p[ci[k]]));
     if (b > kZspBandMax) return BEM_OK;
     b = std::max(b, 1);
+    z->bmax = std::max(z->bmax, b);
+    nband_true += ((int64_t)n * b + 1) & ~(int64_t)1;
+    b = std::max(b, kZspW32 - 1);  // a block's triangle lies in the stored band (k_zsp_invtri)
     ZspObj o;
     o.e0 = e0;
     o.n = n;
@@ -551,7 +624,7 @@ int zsp_prepare(aim_ctx* c, const double* d_verts, const int32_t* d_tris, const 
     z->obj.push_back(o);
     nband += ((int64_t)n * b + 1) & ~(int64_t)1;  // even: 16-byte aligned FP32 slabs
     nwork += (int64_t)n * (2 * b + 1);
-    z->bmax = std::max(z->bmax, b);
+    z->bstore = std::max(z->bstore, b);
     for (int r = 0; r < n; ++r) {
       perm[e0 + r] = e0 + ord[r];
       pos[e0 + ord[r]] = e0 + r;
@@ -561,16 +634,17 @@ int zsp_prepare(aim_ctx* c, const double* d_verts, const int32_t* d_tris, const 
       row[e0 + r + 1] = (int32_t)col.size();
     }
   }
-  // the product kernel's shared memory in FP64: the vector and two slabs
-  if (16 + ((nmax * 16 + 15) & ~(int64_t)15) + 2 * kZspBW * (int64_t)z->bmax * 16 > (int64_t)kZspSmemMax)
+  // room for the FP64 vector and two slabs of 8 columns
+  if (16 + ((nmax * 16 + 15) & ~(int64_t)15) + 2 * kZspW64s * (int64_t)z->bmax * 16 > (int64_t)kZspSmemMax)
     return BEM_OK;
   // worth it only below half the dense bytes (FP32: band tables, diagonal, rows and columns)
-  const int64_t sparse_b = 2 * nband * 8 + (int64_t)c->ne * 8 + (int64_t)col.size() * 12;
+  const int64_t sparse_b = 2 * nband_true * 8 + (int64_t)c->ne * 8 + (int64_t)col.size() * 12;
   if (sparse_b > 4 * dense) return BEM_OK;
   z->nnz = (int64_t)col.size();
   z->nband = nband;
   z->nwork = nwork;
   z->nmax = (int)nmax;
+  z->w64 = zsp_smem_bytes<double2>(z, kZspW64, 2) <= kZspSmemCta ? kZspW64 : kZspW64s;
   BEM_TRY(upload(c, &z->d_obj, z->obj.data(), z->obj.size()));
   BEM_TRY(upload(c, &z->d_perm, perm.data(), perm.size()));
   BEM_TRY(upload(c, &z->d_pos, pos.data(), pos.size()));
@@ -617,6 +691,12 @@ int zsp_factor(aim_ctx* c) {
   for (const ZspObj& o : z->obj) mx = std::max(mx, (int64_t)o.n * o.b);
   k_zsp_extract<<<dim3((unsigned)((mx + 255) / 256), nobj), 256>>>(z->d_obj, z->W, z->L64, z->U64,
                                                                    z->D64, z->L32, z->U32, z->D32);
+  const auto blocks = [&](int w) { return dim3((unsigned)((z->nmax + w - 1) / w), nobj); };
+  k_zsp_invtri<kZspW32, float2><<<blocks(kZspW32), 32>>>(z->d_obj, z->W, z->L32, z->U32);
+  if (z->w64 == kZspW64)
+    k_zsp_invtri<kZspW64, double2><<<blocks(kZspW64), 32>>>(z->d_obj, z->W, z->L64, z->U64);
+  else
+    k_zsp_invtri<kZspW64s, double2><<<blocks(kZspW64s), 32>>>(z->d_obj, z->W, z->L64, z->U64);
   k_round_kv<<<(unsigned)((z->nnz + 255) / 256), 256>>>(z->kv64, z->kv32, z->nnz);
   BEM_CUDA(cudaGetLastError());
   std::vector<int> fail(nobj);

@@ -1,0 +1,50 @@
+"""Block substitutions of the sparse internal operator at the sizes where they can go wrong: edge
+counts that are no multiple of a block, a half-bandwidth next to a block's width (32 columns, whose
+triangle has to fit the stored band) and one above the 128 rows an update pass takes.
+e = Z_s h against the dense Z h of the same context in the same precision, one to four right-hand
+sides. Tolerances: the dropped pairs are below e^-23 = 1e-10 of the kept ones (C64 1e-9, ten times
+that); FP32 products of these lengths round to about 1e-6 (C32 1e-5, the tolerance of the matvec)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2108_03991_gb300 import api, synth  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2108_03991_gb300 import build
+    build.build()
+
+
+def thin_bar():  # 486 edges, half-bandwidth 33 at 20 THz
+    mesh = synth.bar_mesh(0.5, 0.5, 20.0, 0.5)
+    return mesh, synth.grid_box(mesh, 0.5), 2e13
+
+
+def rings(n_theta, n_r):  # two rings at 1 THz
+    return synth.srr_array(2, 2, 1, n_theta=n_theta, n_r=n_r, n_z=1), synth.srr_grid(2), 1e12
+
+
+@pytest.mark.parametrize("make,lo,hi", [(thin_bar, 31, 40), (lambda: rings(61, 2), 97, 128),
+                                        (lambda: rings(80, 3), 160, 192)])
+def test_sparse_against_dense(make, lo, hi):
+    mesh, grid, freq = make()
+    ctx = api.Context(mesh, grid, freq)
+    info = ctx.sparse_internal
+    assert info["objects"] == mesh.nobj and info["on"] and lo <= info["band"] <= hi
+    for prec, tol in ((api.BEM_C64, 1e-9), (api.BEM_C32, 1e-5)):
+        for nrhs in range(1, 5):
+            h = torch.from_numpy(synth.rand_cvec(nrhs * ctx.ne, 31 + nrhs)).to(api.cdtype(prec)).cuda()
+            e = {}
+            for on in (True, False):
+                ctx.internal_sparse(on)
+                e[on] = ctx.internal(h, nrhs=nrhs, prec=prec, want_heq=False)[0].cpu().numpy()
+            for s, d in zip(np.split(e[True], mesh.nobj * nrhs), np.split(e[False], mesh.nobj * nrhs)):
+                assert np.linalg.norm(s - d) <= tol * np.linalg.norm(d)
+    assert not ctx.internal_sparse(True)["wait_timed_out"]
+    ctx.close()
