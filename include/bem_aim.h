@@ -243,13 +243,12 @@ int aim_conv(aim_ctx* ctx, const void* sigma, void* phi, int ncomp, int prec, vo
 /* y_i = A_i x_i for nblk square blocks (Sec. II-C block-diagonal Z, Y_eq). n: HOST array of
  * block sizes. A: DEVICE array, block i row-major with leading dimension ld_i = n_i rounded up
  * to a multiple of 4, blocks one after another (offsets sum of n_j*ld_j). x, y: nrhs vectors of
- * sum n_i each. */
+ * sum n_i each. The table of blocks travels with the launch: nothing is allocated or copied. */
 int bem_blockdiag_gemv(int nblk, const int32_t* n, const void* A, const void* x, void* y,
                        int nrhs, int prec, void* stream);
 
 /* The same product as bem_blockdiag_gemv for callers that cannot allocate device memory (the
- * paper has no counterpart). bem_blockdiag_gemv allocates its row-panel work list on every
- * call; this variant allocates nothing and keeps the list in a fixed 1 MiB device array built
+ * paper has no counterpart). It keeps its list of row panels in a fixed 1 MiB device array built
  * into the library, which every GPU that loads the library holds until exit. It takes the
  * same arguments and gives the same result. Limit: at most 32768 panels of 16 rows, i.e. the
  * sum over blocks of ceil(n_i / 16) <= 32768 (up to 524,288 rows); larger inputs return

@@ -320,54 +320,21 @@ int bem_blockdiag_gemv(int nblk, const int32_t* n, const void* A, const void* x,
     set_error("bem_blockdiag_gemv: bad arguments");
     return BEM_EINVAL;
   }
-  std::vector<int32_t> nn(n, n + nblk), xo(nblk), ld(nblk);
-  std::vector<int64_t> off(nblk);
-  int64_t o = 0;
-  int32_t xs = 0;
+  int64_t rows = 0;
   for (int i = 0; i < nblk; ++i) {
-    if (nn[i] < 1) {
+    if (n[i] < 1) {
       set_error("bem_blockdiag_gemv: block sizes must be positive");
       return BEM_EINVAL;
     }
-    ld[i] = (int32_t)round_up(nn[i], 4);
-    off[i] = o;
-    xo[i] = xs;
-    o += (int64_t)nn[i] * ld[i];
-    xs += nn[i];
+    rows += n[i];
   }
-  int dev = 0, nsm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  // the persistent byte-balanced launch of the context's plain internal products (4-6 CTAs per
-  // SM, rows of all blocks cut into equal-byte ranges), with the default shape (no autotuning)
-  std::vector<RowInfo> rows;
-  std::vector<int2> segs;
-  std::vector<int32_t> cseg;
-  double ratio = 0;
-  const int ncta = nsm * kGemvCtasPerSm;
-  build_gemv_plan(nn, off, ld, ncta, &rows, &segs, &cseg, &ratio);
-  const size_t b0 = rows.size() * sizeof(RowInfo), b1 = segs.size() * sizeof(int2),
-               b2 = cseg.size() * sizeof(int32_t);
-  const size_t o1 = round_up(b0, 256), o2 = o1 + round_up(b1, 256);
-  char* d = nullptr;
+  if (rows > INT32_MAX) {
+    set_error("bem_blockdiag_gemv: more than 2^31 - 1 rows");
+    return BEM_EINVAL;
+  }
   cudaStream_t s = (cudaStream_t)stream;
-  BEM_CUDA(cudaMallocAsync((void**)&d, o2 + b2, s));
-  BEM_CUDA(cudaMemcpyAsync(d, rows.data(), b0, cudaMemcpyHostToDevice, s));
-  BEM_CUDA(cudaMemcpyAsync(d + o1, segs.data(), b1, cudaMemcpyHostToDevice, s));
-  BEM_CUDA(cudaMemcpyAsync(d + o2, cseg.data(), b2, cudaMemcpyHostToDevice, s));
-  GemvPlan p;
-  p.rows = (RowInfo*)d;
-  p.segs = (int2*)(d + o1);
-  p.cta_seg = (int32_t*)(d + o2);
-  p.ncta = ncta;
-  p.nrows = (int)rows.size();
-  int rc = prec == BEM_C32
-               ? run_gemv_plan<float>(p, (const float2*)A, (const float2*)x, (float2*)y, nrhs, xs, nullptr, s)
-               : run_gemv_plan<double>(p, (const double2*)A, (const double2*)x, (double2*)y, nrhs, xs, nullptr, s);
-  cudaFreeAsync(d, s);
-  // the host vectors must outlive the asynchronous copies
-  cudaStreamSynchronize(s);
-  return rc;
+  return prec == BEM_C32 ? run_gemv_blocks<float>(nblk, n, (const float2*)A, (const float2*)x, (float2*)y, nrhs, s)
+                         : run_gemv_blocks<double>(nblk, n, (const double2*)A, (const double2*)x, (double2*)y, nrhs, s);
 }
 
 int64_t aim_export(const aim_ctx* c, int what, int index, void* out, int64_t cap) {

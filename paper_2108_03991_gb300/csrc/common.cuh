@@ -383,6 +383,10 @@ template <typename R>
 int run_gemv(const GemvTask* d_tasks, int ntasks, const typename C2<R>::T* A,
              const typename C2<R>::T* x, typename C2<R>::T* y, int nrhs, int64_t vstride,
              const typename C2<R>::T* hsub, cudaStream_t s);
+// y_i = A_i x_i of a caller's packed blocks (sizes n on the host), nothing allocated or copied
+template <typename R>
+int run_gemv_blocks(int nblk, const int32_t* n, const typename C2<R>::T* A,
+                    const typename C2<R>::T* x, typename C2<R>::T* y, int nrhs, cudaStream_t s);
 template <typename R>
 int run_gemv_mr(const GemvPlan& p, const typename C2<R>::T* A, const typename C2<R>::T* x,
                 typename C2<R>::T* y, int nrhs, int64_t vstride, const typename C2<R>::T* hsub,

@@ -8,6 +8,8 @@
 //   a = W phi + L^A_NR j        ;  y1 = j k0 a + I_x e - (F D)^T p  (one warp per edge)
 // Sec. III-A item 1 (Eq. AIM_L) gives L = L_NR + W H P; Sec. II-C (Eq. Cdef) gives the
 // combination C = (-j k0 L^A Y + I_x/eta0) Z.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace bem {
@@ -27,8 +29,10 @@ template <> struct Vec16<float> { typedef float4 T; static constexpr int kCplx =
 template <> struct Vec16<double> { typedef double2 T; static constexpr int kCplx = 1; };
 
 // acc[r] += sum over the 16-byte vectors [v0, v1) of one row of A (lane-strided) times x_r.
-// U vectors per lane are loaded before any is used, so each lane keeps U loads in flight.
-template <typename R, int NRHS, int U>
+// U vectors per lane are loaded before any is used, so each lane keeps U loads in flight. PAIR: the
+// two entries of an FP32 vector are summed before they meet the accumulator, which halves the
+// length of the lane's chain of roundings.
+template <typename R, int NRHS, int U, bool PAIR = false>
 __device__ __forceinline__ void dot_range(const typename Vec16<R>::T* __restrict__ arow,
                                           const typename C2<R>::T* __restrict__ xb, int n, int v0,
                                           int v1, int64_t vstride, int lane,
@@ -47,8 +51,18 @@ __device__ __forceinline__ void dot_range(const typename Vec16<R>::T* __restrict
       for (int r = 0; r < NRHS; ++r) {
         if (x16[r] && col + 1 < n) {
           const float4 q = __ldg(reinterpret_cast<const float4*>(xb + r * vstride + col));
-          cfma(acc[r], a0, mk(q.x, q.y));
-          cfma(acc[r], a1, mk(q.z, q.w));
+          if constexpr (PAIR) {
+            auto t = cmul(a0, mk(q.x, q.y));
+            cfma(t, a1, mk(q.z, q.w));
+            acc[r] = cadd(acc[r], t);
+          } else {
+            cfma(acc[r], a0, mk(q.x, q.y));
+            cfma(acc[r], a1, mk(q.z, q.w));
+          }
+        } else if (PAIR) {
+          auto t = cmul(a0, __ldg(xb + r * vstride + col));
+          if (col + 1 < n) cfma(t, a1, __ldg(xb + r * vstride + col + 1));
+          acc[r] = cadd(acc[r], t);
         } else {
           cfma(acc[r], a0, __ldg(xb + r * vstride + col));
           if (col + 1 < n) cfma(acc[r], a1, __ldg(xb + r * vstride + col + 1));
@@ -75,17 +89,40 @@ __device__ __forceinline__ void dot_range(const typename Vec16<R>::T* __restrict
 // One row of the product, one warp: acc[r] = sum_k A[row, k] x_r[k]. Rows are streamed with
 // 16-byte loads (two complex FP32 or one complex FP64 per load), evict-first so the streamed
 // matrix does not displace the vectors in L2; x is read through the read-only path (L1).
-template <typename R, int NRHS, int U = 4>
+template <typename R, int NRHS, int U = 4, bool PAIR = false>
 __device__ __forceinline__ void row_dot(const typename C2<R>::T* __restrict__ arow,
                                         const typename C2<R>::T* __restrict__ xb, int n,
                                         int64_t vstride, int lane, typename C2<R>::T* acc) {
   constexpr int CP = Vec16<R>::kCplx;
 #pragma unroll
   for (int r = 0; r < NRHS; ++r) acc[r] = czero<typename C2<R>::T>();
-  dot_range<R, NRHS, U>(reinterpret_cast<const typename Vec16<R>::T*>(arow), xb, n, 0,
+  dot_range<R, NRHS, U, PAIR>(reinterpret_cast<const typename Vec16<R>::T*>(arow), xb, n, 0,
                         (n + CP - 1) / CP, vstride, lane, acc);
 #pragma unroll
   for (int r = 0; r < NRHS; ++r) acc[r] = warp_sum(acc[r]);
+}
+
+// one task (a run of rows of one block) by the NW warps of a CTA, a row at a time
+template <typename R, int NRHS, int U, int NW, bool PAIR = false>
+__device__ __forceinline__ void gemv_task(const GemvTask& t, const typename C2<R>::T* __restrict__ A,
+                                          const typename C2<R>::T* __restrict__ x,
+                                          typename C2<R>::T* __restrict__ y, int64_t vstride,
+                                          const typename C2<R>::T* __restrict__ hsub) {
+  typedef typename C2<R>::T V;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const V* xb = x + t.xoff;
+  for (int rr = warp; rr < t.nrows; rr += NW) {
+    const int row = t.row0 + rr;
+    V acc[NRHS];
+    row_dot<R, NRHS, U, PAIR>(A + t.aoff + (int64_t)row * t.ld, xb, t.n, vstride, lane, acc);
+#pragma unroll
+    for (int r = 0; r < NRHS; ++r) {
+      if (lane == 0) {
+        int64_t o = r * vstride + t.xoff + row;
+        y[o] = hsub ? csub(hsub[o], acc[r]) : acc[r];
+      }
+    }
+  }
 }
 
 // Task-list form: one CTA per task (a run of rows of one block), NW warps taking the rows in
@@ -97,22 +134,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_gemv(const GemvTask* __restri
                                               const typename C2<R>::T* __restrict__ x,
                                               typename C2<R>::T* __restrict__ y, int64_t vstride,
                                               const typename C2<R>::T* __restrict__ hsub) {
-  typedef typename C2<R>::T V;
-  const GemvTask t = tasks[blockIdx.x];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const V* xb = x + t.xoff;
-  for (int rr = warp; rr < t.nrows; rr += NW) {
-    const int row = t.row0 + rr;
-    V acc[NRHS];
-    row_dot<R, NRHS, U>(A + t.aoff + (int64_t)row * t.ld, xb, t.n, vstride, lane, acc);
-#pragma unroll
-    for (int r = 0; r < NRHS; ++r) {
-      if (lane == 0) {
-        int64_t o = r * vstride + t.xoff + row;
-        y[o] = hsub ? csub(hsub[o], acc[r]) : acc[r];
-      }
-    }
-  }
+  gemv_task<R, NRHS, U, NW>(tasks[blockIdx.x], A, x, y, vstride, hsub);
 }
 
 // Several right-hand sides at once: each warp takes RB (2 or 4) rows of its task and NR right-hand
@@ -121,16 +143,14 @@ __global__ void __launch_bounds__(NW * 32, MINB) k_gemv(const GemvTask* __restri
 // warps per task of at most RB NW rows; y_r = A x_r, or hsub_r - A x_r. x is read as 8-byte
 // complex pairs (its slices need not be 16-byte aligned); an odd row length masks the last
 // pair's second entry.
-template <typename R, int NR, int NW, int RB>
-__global__ void __launch_bounds__(NW * 32) k_gemv_mr(const GemvTask* __restrict__ tasks,
-                                                     const typename C2<R>::T* __restrict__ A,
-                                                     const typename C2<R>::T* __restrict__ x,
-                                                     typename C2<R>::T* __restrict__ y, int64_t vstride,
-                                                     const typename C2<R>::T* __restrict__ hsub) {
+template <typename R, int NR, int RB, bool PAIR = false>
+__device__ __forceinline__ void gemv_mr_task(const GemvTask& t, const typename C2<R>::T* __restrict__ A,
+                                             const typename C2<R>::T* __restrict__ x,
+                                             typename C2<R>::T* __restrict__ y, int64_t vstride,
+                                             const typename C2<R>::T* __restrict__ hsub) {
   typedef typename C2<R>::T V;
   typedef typename Vec16<R>::T L16;  // 16 bytes: two complex FP32 or one complex FP64
   constexpr int CP = Vec16<R>::kCplx;
-  const GemvTask t = tasks[blockIdx.x];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r0 = t.row0 + warp * RB;
   const int nr = min(RB, t.row0 + t.nrows - r0);
@@ -157,6 +177,22 @@ __global__ void __launch_bounds__(NW * 32) k_gemv_mr(const GemvTask* __restrict_
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (v + 32 * u >= nv) break;
+      if constexpr (PAIR && CP == 2) {  // as in dot_range
+        const int col = 2 * (v + 32 * u);
+        const bool two = col + 1 < t.n;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const V x0 = __ldg(xb + r * vstride + col);
+          const V x1 = two ? __ldg(xb + r * vstride + col + 1) : czero<V>();
+#pragma unroll
+          for (int k = 0; k < RB; ++k) {
+            V p = cmul(mk(a[u][k].x, a[u][k].y), x0);
+            if (two) cfma(p, mk(a[u][k].z, a[u][k].w), x1);
+            acc[k][r] = cadd(acc[k][r], p);
+          }
+        }
+        continue;
+      }
 #pragma unroll
       for (int q = 0; q < CP; ++q) {
         const int col = (v + 32 * u) * CP + q;
@@ -192,6 +228,15 @@ __global__ void __launch_bounds__(NW * 32) k_gemv_mr(const GemvTask* __restrict_
       y[o] = hsub ? csub(hsub[o], out) : out;
     }
   }
+}
+
+template <typename R, int NR, int NW, int RB>
+__global__ void __launch_bounds__(NW * 32) k_gemv_mr(const GemvTask* __restrict__ tasks,
+                                                     const typename C2<R>::T* __restrict__ A,
+                                                     const typename C2<R>::T* __restrict__ x,
+                                                     typename C2<R>::T* __restrict__ y, int64_t vstride,
+                                                     const typename C2<R>::T* __restrict__ hsub) {
+  gemv_mr_task<R, NR, RB>(tasks[blockIdx.x], A, x, y, vstride, hsub);
 }
 
 template <typename R>
@@ -637,6 +682,145 @@ template int run_gemv<float>(const GemvTask*, int, const float2*, const float2*,
                              int64_t, const float2*, cudaStream_t);
 template int run_gemv<double>(const GemvTask*, int, const double2*, const double2*, double2*, int,
                               int64_t, const double2*, cudaStream_t);
+
+// ---------------------------------------------------------------------------------------
+// block-diagonal product of a caller's blocks, no set-up
+// ---------------------------------------------------------------------------------------
+// The blocks' table travels as a kernel argument (no allocation, no copy, nothing to wait for);
+// a CTA finds its task, RT rows of one block, by bisection over the blocks' first tasks (uniform
+// reads of the argument). The tasks are those of the task-list form, which the set-up's tuner
+// finds the fastest on most structures: small, handed out by the hardware, largest blocks first.
+// A persistent launch over a table of all rows, built and uploaded on each call, was the form
+// before. FP32, one right-hand side: 1,024 blocks of 912 (6.8 GB) 3,445 -> 960 us, 100 of them 543
+// -> 97, 300 of 1-700 629 -> 66, 4 of 120 216 -> 17 us (the host's call); FP64, 100 of 912 1,199 ->
+// 762 us, then at the FP64 rate.
+template <int CAP> struct BlkTab {
+  int nblk;
+  uint32_t first[CAP];  // first task of block b
+  uint32_t aoff[CAP];   // element offset of the block / 4
+  int32_t xoff[CAP];    // first unknown
+  int32_t n[CAP];
+};
+template <int CAP> __device__ __forceinline__ GemvTask blk_task(const BlkTab<CAP>& tab, int rt) {
+  int lo = 0, hi = tab.nblk;  // first[lo] <= blockIdx.x < first[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (tab.first[mid] <= blockIdx.x) lo = mid;
+    else hi = mid;
+  }
+  GemvTask t;
+  t.aoff = 4 * (int64_t)tab.aoff[lo];
+  t.xoff = tab.xoff[lo];
+  t.n = tab.n[lo];
+  t.ld = (t.n + 3) & ~3;
+  t.row0 = (int)(blockIdx.x - tab.first[lo]) * rt;
+  t.nrows = min(rt, t.n - t.row0);
+  t.sel = 0;
+  return t;
+}
+template <typename R, int CAP>
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 16 : 0)
+    k_gemv_blk(const __grid_constant__ BlkTab<CAP> tab, const typename C2<R>::T* __restrict__ A,
+               const typename C2<R>::T* __restrict__ x, typename C2<R>::T* __restrict__ y) {
+  gemv_task<R, 1, 4, 4, true>(blk_task(tab, 4), A, x, y, 0, nullptr);
+}
+template <typename R, int NR, int CAP>
+__global__ void __launch_bounds__(128)
+    k_gemv_blk_mr(const __grid_constant__ BlkTab<CAP> tab, const typename C2<R>::T* __restrict__ A,
+                  const typename C2<R>::T* __restrict__ x, typename C2<R>::T* __restrict__ y,
+                  int64_t vstride) {
+  gemv_mr_task<R, NR, 4, true>(blk_task(tab, 16), A, x, y, vstride, nullptr);
+}
+
+template <typename R, int CAP>
+static int launch_blk(const BlkTab<CAP>& tab, unsigned ntask, const typename C2<R>::T* A,
+                      const typename C2<R>::T* x, typename C2<R>::T* y, int nrhs, int64_t vs,
+                      cudaStream_t s) {
+  if (nrhs == 1) {
+    k_gemv_blk<R, CAP><<<ntask, 128, 0, s>>>(tab, A, x, y);
+  } else {
+    for (int r0 = 0; r0 < nrhs; r0 += 4) {
+      const int64_t o = r0 * vs;
+      switch (std::min(4, nrhs - r0)) {
+        case 1: k_gemv_blk_mr<R, 1, CAP><<<ntask, 128, 0, s>>>(tab, A, x + o, y + o, vs); break;
+        case 2: k_gemv_blk_mr<R, 2, CAP><<<ntask, 128, 0, s>>>(tab, A, x + o, y + o, vs); break;
+        case 3: k_gemv_blk_mr<R, 3, CAP><<<ntask, 128, 0, s>>>(tab, A, x + o, y + o, vs); break;
+        default: k_gemv_blk_mr<R, 4, CAP><<<ntask, 128, 0, s>>>(tab, A, x + o, y + o, vs); break;
+      }
+    }
+  }
+  BEM_CUDA(cudaGetLastError());
+  return BEM_OK;
+}
+
+// sizes n[nblk] on the host, blocks packed as in bem_blockdiag_gemv; one launch (per four
+// right-hand sides) for every 1,984 blocks: a kernel's arguments are limited to 32,764 bytes
+template <typename R>
+int run_gemv_blocks(int nblk, const int32_t* n, const typename C2<R>::T* A,
+                    const typename C2<R>::T* x, typename C2<R>::T* y, int nrhs, cudaStream_t s) {
+  constexpr int kSmall = 64, kLarge = 1984;
+  static_assert(sizeof(BlkTab<kLarge>) + 64 <= 32764, "kernel argument size");
+  const int rt = nrhs == 1 ? 4 : 16;
+  int64_t vs = 0;
+  for (int i = 0; i < nblk; ++i) vs += n[i];
+  std::vector<int> order;
+  std::vector<int64_t> ao, xo;
+  int64_t a0 = 0, x0 = 0;
+  for (int b0 = 0; b0 < nblk;) {
+    // the chunk's blocks, offsets counted from its start (aoff / 4 in 32 bits)
+    ao.clear();
+    xo.clear();
+    int64_t a = 0, xx = 0, tasks = 0;
+    int b1 = b0;
+    for (; b1 < nblk && b1 - b0 < kLarge; ++b1) {
+      const int64_t t = (n[b1] + rt - 1) / rt;
+      if (b1 > b0 && (a / 4 > UINT32_MAX || tasks + t > INT32_MAX)) break;
+      ao.push_back(a);
+      xo.push_back(xx);
+      a += (int64_t)n[b1] * round_up(n[b1], 4);
+      xx += n[b1];
+      tasks += t;
+    }
+    const int nb = b1 - b0;
+    order.resize(nb);
+    bool sorted = true;
+    for (int i = 0; i < nb; ++i) {
+      order[i] = i;
+      sorted = sorted && (i == 0 || n[b0 + i] <= n[b0 + i - 1]);
+    }
+    if (!sorted)
+      std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return n[b0 + p] > n[b0 + q]; });
+    auto fill = [&](auto& tab) {
+      tab.nblk = nb;
+      uint32_t t = 0;
+      for (int i = 0; i < nb; ++i) {
+        const int b = order[i];
+        tab.first[i] = t;
+        tab.aoff[i] = (uint32_t)(ao[b] / 4);
+        tab.xoff[i] = (int32_t)xo[b];
+        tab.n[i] = n[b0 + b];
+        t += (uint32_t)((n[b0 + b] + rt - 1) / rt);
+      }
+    };
+    if (nb <= kSmall) {
+      BlkTab<kSmall> tab;
+      fill(tab);
+      BEM_TRY((launch_blk<R, kSmall>(tab, (unsigned)tasks, A + a0, x + x0, y + x0, nrhs, vs, s)));
+    } else {
+      BlkTab<kLarge> tab;
+      fill(tab);
+      BEM_TRY((launch_blk<R, kLarge>(tab, (unsigned)tasks, A + a0, x + x0, y + x0, nrhs, vs, s)));
+    }
+    a0 += a;
+    x0 += xx;
+    b0 = b1;
+  }
+  return BEM_OK;
+}
+template int run_gemv_blocks<float>(int, const int32_t*, const float2*, const float2*, float2*, int,
+                                    cudaStream_t);
+template int run_gemv_blocks<double>(int, const int32_t*, const double2*, const double2*, double2*,
+                                     int, cudaStream_t);
 
 // ---------------------------------------------------------------------------------------
 // projection P (Sec. III-A item 1): gather form, no atomics, deterministic
