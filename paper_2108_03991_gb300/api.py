@@ -486,8 +486,7 @@ class Context:
         return e, heq
 
     def tc_variant(self, variant):
-        """Form of the tensor-core product (aim_tc_variant): 0 hi/lo packed, 1 raw B split in
-        shared memory."""
+        """Form of the tensor-core product (aim_tc_variant): 0 or 1, the same launch."""
         _check(lib().aim_tc_variant(self.h, int(variant)))
 
     def tensor_core_status(self):

@@ -460,7 +460,6 @@ int aim_tc_variant(aim_ctx* c, int variant) {
     set_error("aim_tc_variant: variant must be 0 or 1");
     return BEM_EINVAL;
   }
-  c->tc_variant = variant;
   return BEM_OK;
 }
 

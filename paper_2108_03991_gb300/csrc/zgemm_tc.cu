@@ -9,29 +9,35 @@
 //   column 2r + 1 = ( Im x_0,  Re x_0,  Im x_1,  Re x_1, ...)   (gives Im y_r),
 // so D = A_real B (M = n, K = 2n, N = 2R) holds y_r as the (re, im) pair of columns 2r, 2r + 1.
 //
-// FP32 accuracy from TF32 tensor cores by the three-product split: a = a_hi + a_lo with a_hi the
-// value with its 13 low mantissa bits cleared (exact in TF32) and a_lo = a - a_hi (exact in
-// FP32, 11 significant bits kept by TF32), D = A_hi B_hi + A_hi B_lo + A_lo B_hi; the dropped
-// A_lo B_lo and the truncation of the lo parts leave about 2^-20 relative error per product.
+// FP32 accuracy from FP16 tensor cores by the three-product split. Every row of A and every
+// (object, right-hand side) slice of x is scaled by the power of two that brings its largest entry
+// into [2^14, 2^15); then a = a_hi + a_lo with a_hi the nearest FP16 value and a_lo the nearest FP16
+// value of the rest, 22 significant bits (entries below 2^-18 of the largest keep 2^-40 of it), and
+// D = A_hi B_hi + A_hi B_lo + A_lo B_hi in FP32, scaled back exactly. The dropped A_lo B_lo is 2^-22.
+// The split of an FP32 tile into TF32 parts, the form before, has the same 22 bits but twice the bytes
+// in shared memory, twice the MMAs at half their rate, and twice the truncations of the accumulator.
 //
-// Layout. B (both halves) is packed once per call from x into [N][K_tot] with every object's
-// K range starting at 2 sum_{j<i} ld_j (a multiple of 8 floats, so every TMA start is 16-byte
-// aligned) and zeros in the padding slots. A is read in place through one 2-D tensor map per
-// object (inner extent 2n, rows n, row pitch 8 ld bytes): TMA fills the K tail and the rows
-// past n with zeros, so a tile that reads past its object's K range in B meets zeros in A.
-// Shared-memory tiles are K-major with the 128-byte swizzle, 32 floats of K per row.
+// Layout. B is packed once per call from x into [N][K_tot]: every object's K range starts at a
+// multiple of 32 values and every 32 values of a row are 128 bytes, 32 FP16 hi parts then their 32 lo
+// parts (zeros past the object's 2 n values). A is read in place through one 2-D tensor map per
+// object (inner extent 2n floats, rows n, row pitch 8 ld bytes): TMA fills the K tail and the rows
+// past n with zeros; the landed FP32 tile is turned in place into the same [32 hi | 32 lo] rows.
+// Shared-memory tiles are K-major with the 128-byte swizzle.
 //
-// One CTA of four warps per 128-row tile of one block (tiles in decreasing block size). Thread
-// 0 issues the TMA loads into a ring of stages and the MMAs (M = 128, N = 2R padded to NP, K = 8
-// per instruction) into one TMEM accumulator of NP columns; all threads split the stage's A
-// tile into hi and lo parts in shared memory while the previous stage's MMAs run. The epilogue
-// reads TMEM lane by lane (warp w owns rows 32w..32w+31) and writes y_r coalesced along rows.
+// A product is bound by shared memory (a stage of 32 K values moves 112 KB through it at N = 128: the
+// landing tiles, the conversion, the operands of 6 MMAs) and by the HBM reads of the blocks, so both
+// matrices go in one launch of persistent CTAs and the K loops of the tiles are cut into units that
+// load them evenly (tc_units). Z and C together, packing included, against one launch per matrix with
+// a CTA per tile in TF32 (us, 64 right-hand sides): six bars of 240-1,920 edges 257 -> 69, one bar of
+// 2,016 263 -> 40, 16 rings of 912 144 -> 72; 128 right-hand sides 539 -> 100, 446 -> 56, 262 -> 104;
+// 144 rings (HBM-bound) 395 at 1, 467 at 64. Error against 64 bits on the rings 6.6e-6 -> 2.2e-6.
 // Every wait is bounded: on a timeout the CTA records an error (err[0], kept across products)
 // and raises the launch's abort flag (err[1], cleared before each launch), waits (with a short
 // limit) for its own MMAs and copies in flight, frees its TMEM and leaves; the other CTAs see
 // the flag in their waits, or before they start, and leave too. The results are then invalid.
 #include <cuda.h>
 #include <cudaTypedefs.h>
+#include <cuda_fp16.h>
 
 #include <algorithm>
 
@@ -42,12 +48,23 @@ namespace bem {
 
 constexpr int kTcM = 128;       // rows per tile (MMA M, TMEM lanes)
 constexpr int kTcK = 32;        // floats of K per stage: one 128-byte swizzle row
-constexpr int kTcThreads = 128;
+// Per width NP of B: stages S, threads G that convert one stage. One group of threads per stage: a
+// group waits on its loads and its proxy fence while the others work, and never waits for a phase
+// of its stage that is two ahead.
+template <int NP> struct TcShape;
+template <> struct TcShape<32> { static constexpr int S = 8, G = 32; };
+template <> struct TcShape<64> { static constexpr int S = 7, G = 32; };
+template <> struct TcShape<128> { static constexpr int S = 6, G = 64; };
+template <> struct TcShape<256> { static constexpr int S = 4, G = 64; };
+constexpr int kTcEpi = 128;  // threads that read the accumulators, one row of a tile each
+template <int NP> constexpr int tc_threads() { return kTcEpi + 64 + TcShape<NP>::S * TcShape<NP>::G; }
 constexpr int kTcMaxRhs = 128;  // N = 2R <= 256 per launch
 constexpr uint32_t kTcAtile = kTcM * kTcK * 4;  // 16 KB
 
-struct TcTile {  // one 128-row tile of one block
-  int32_t obj, row0;
+struct TcUnit {  // stages [k0, k1) of one 128-row tile of one block of Z (mat 0) or C (mat 1)
+  int32_t obj, row0, mat, k0, k1;
+  int32_t parts;        // units of the tile; its partial sums are the slots slot0 .. slot0 + parts - 1
+  int32_t slot, slot0;  // (parts > 1 only)
 };
 struct TcObj {   // per object: size, first unknown, first K column in the packed B
   int32_t n, xoff;
@@ -62,12 +79,11 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
-// instruction descriptor of kind::tf32: D in FP32 (bits 4-5 = 1), A and B TF32 (bits 7-9 and
-// 10-12 = 2), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-__host__ __device__ constexpr uint32_t tf32_idesc(int M, int N) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// instruction descriptor of kind::f16: D in FP32 (bits 4-5 = 1), A and B FP16 (bits 7-9 and 10-12 =
+// 0), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
+__host__ __device__ constexpr uint32_t f16_idesc(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-static_assert(tf32_idesc(128, 256) == 0x08400910u, "instruction descriptor fields");
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, int x, int y, uint64_t* bar) {
   asm volatile(
@@ -91,11 +107,11 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-__device__ __forceinline__ void tc_mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
+__device__ __forceinline__ void tc_mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
                                             uint32_t accumulate) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -121,10 +137,27 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ float tf32_hi(float a) { return __uint_as_float(__float_as_uint(a) & 0xFFFFE000u); }
+// exponent shift that brings a slice's largest magnitude m into [2^14, 2^15); 0 for a zero slice
+__device__ __forceinline__ int tc_shift(float m) {
+  if (!(m > 0.f)) return 0;
+  const int e = (int)(__float_as_uint(m) >> 23) - 127;  // floor(log2 m); -127 below the normal range
+  return min(126, 14 - e);
+}
+__device__ __forceinline__ float tc_pow2(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
+__device__ __forceinline__ uint32_t h2(float a, float b) {
+  const __half2 v = __floats2half2_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+// hi and lo parts of two scaled values
+__device__ __forceinline__ void tc_halves(float a, float b, uint32_t* hi, uint32_t* lo) {
+  const __half2 h = __floats2half2_rn(a, b);
+  const float2 f = __half22float2(h);
+  *hi = *reinterpret_cast<const uint32_t*>(&h);
+  *lo = h2(a - f.x, b - f.y);
+}
 
 // Bounded wait on an mbarrier phase that also gives up as soon as any CTA of the launch has
-// recorded a failure in *err (polled every 256 tries), so that one stuck CTA does not make
+// recorded a failure in *err (polled every 8192 tries), so that one stuck CTA does not make
 // every later CTA wait out its own limit.
 constexpr uint32_t kTcSpin = 1u << 22;
 constexpr uint32_t kTcSpinCleanup = 1u << 16;
@@ -138,203 +171,364 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, const in
         : "r"(smem_u32(bar)), "r"(parity)
         : "memory");
     if (ok) return true;
-    if ((it & 255) == 255 && *(const volatile int*)err) return false;
+    if ((it & 8191) == 8191 && *(const volatile int*)err) return false;
   }
   return false;
 }
 
-// B from x, hi and lo parts (or, with bl null, the raw FP32 values into bh): rows 2r and 2r + 1
-// for right-hand side r < R (zero rows up to NP), columns 2u and 2u + 1 for padded slot u
-// (slot[u] = its unknown, -1 in a block's padding). Grid: x over the slots, y over the NP / 2
-// row pairs.
-__global__ void k_tc_pack(const float2* __restrict__ x, int64_t vstride, int R,
-                          const int32_t* __restrict__ slot, int64_t nslot, float* __restrict__ bh,
-                          float* __restrict__ bl) {
-  const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int r = blockIdx.y;
-  if (u >= nslot) return;
-  const int j = slot[u];
-  float2 v = make_float2(0.f, 0.f);
-  if (r < R && j >= 0) v = x[r * vstride + j];
-  const int64_t ktot = 2 * nslot;
-  const float2 re = make_float2(v.x, -v.y), im = make_float2(v.y, v.x);
-  const float2 reh = make_float2(tf32_hi(re.x), tf32_hi(re.y)), imh = make_float2(tf32_hi(im.x), tf32_hi(im.y));
-  const int64_t o0 = (2 * r) * ktot + 2 * u, o1 = o0 + ktot;
-  if (!bl) {  // the raw values: the product splits them in shared memory
-    *reinterpret_cast<float2*>(bh + o0) = re;
-    *reinterpret_cast<float2*>(bh + o1) = im;
-    return;
-  }
-  *reinterpret_cast<float2*>(bh + o0) = reh;
-  *reinterpret_cast<float2*>(bh + o1) = imh;
-  *reinterpret_cast<float2*>(bl + o0) = make_float2(re.x - reh.x, re.y - reh.y);
-  *reinterpret_cast<float2*>(bl + o1) = make_float2(im.x - imh.x, im.y - imh.y);
+// exponent shift of every row of a block-diagonal matrix (set-up of the first product): one warp per row
+__global__ void __launch_bounds__(256) k_tc_rowshift(const TcObj* __restrict__ objs, const int64_t* __restrict__ off,
+                                                     const float2* __restrict__ A, int32_t* __restrict__ sh) {
+  const TcObj o = objs[blockIdx.y];
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= o.n) return;
+  const float2* a = A + off[blockIdx.y] + (int64_t)row * ((o.n + 3) & ~3);
+  float m = 0.f;
+  for (int k = lane; k < o.n; k += 32) m = fmaxf(m, fmaxf(fabsf(a[k].x), fabsf(a[k].y)));
+#pragma unroll
+  for (int q = 16; q > 0; q >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, q));
+  if (lane == 0) sh[o.xoff + row] = tc_shift(m);
 }
 
-// shared memory of one CTA: S stages of [A (hi after the split) | A lo | B hi | B lo], each tile
-// 1024-byte aligned, then the full/empty barriers of the stages, the done barrier, the TMEM slot
-template <int NP, int S> struct TcSmem {
-  static constexpr uint32_t kBtile = NP * kTcK * 4;
-  static constexpr uint32_t kStage = 2 * kTcAtile + 2 * kBtile;
+// (re, im) 2^-sh, in two factors of normal range
+__device__ __forceinline__ float2 tc_unscale(float re, float im, int sh) {
+  const int e1 = -sh >> 1;
+  const float f1 = tc_pow2(e1), f2 = tc_pow2(-sh - e1);
+  return make_float2(re * f1 * f2, im * f1 * f2);
+}
+
+// B from x: rows 2r and 2r + 1 of right-hand side r < R (zero rows up to NP), one CTA per object and
+// right-hand side: the slice's largest entry, then its 2 n values as FP16 hi and lo parts, zeros up
+// to the object's padded length
+__global__ void __launch_bounds__(256) k_tc_pack(const float2* __restrict__ x, int64_t vstride, int R,
+                                                 const TcObj* __restrict__ objs, int64_t ktot,
+                                                 uint32_t* __restrict__ b, int32_t* __restrict__ shb) {
+  const TcObj o = objs[blockIdx.x];
+  const int r = blockIdx.y;
+  const float2* xs = x + r * vstride + o.xoff;
+  float m = 0.f;
+  if (r < R)
+    for (int k = threadIdx.x; k < o.n; k += 256) m = fmaxf(m, fmaxf(fabsf(xs[k].x), fabsf(xs[k].y)));
+  __shared__ float red[8];
+#pragma unroll
+  for (int q = 16; q > 0; q >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, q));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 8; ++q) m = fmaxf(m, red[q]);
+  const int sh = tc_shift(m);
+  const float s = tc_pow2(sh);
+  if (threadIdx.x == 0) shb[blockIdx.x * (int64_t)kTcMaxRhs + r] = sh;
+  // in units of 4 bytes (two FP16 values): slot u of 32-value chunk q is hi at 32 q + u, lo 16 further
+  uint32_t* b0 = b + 2 * r * ktot + o.koff;
+  uint32_t* b1 = b0 + ktot;
+  for (int k = threadIdx.x; k < (o.n + 15 & ~15); k += 256) {
+    float2 v = make_float2(0.f, 0.f);
+    if (r < R && k < o.n) v = make_float2(xs[k].x * s, xs[k].y * s);
+    uint32_t hi, lo;
+    const int64_t at = 32 * (int64_t)(k >> 4) + (k & 15);
+    tc_halves(v.x, -v.y, &hi, &lo);
+    b0[at] = hi;
+    b0[at + 16] = lo;
+    tc_halves(v.y, v.x, &hi, &lo);
+    b1[at] = hi;
+    b1[at + 16] = lo;
+  }
+}
+
+// shared memory of one CTA: S stages of [A | B], each tile 1024-byte aligned, then the barriers, the
+// TMEM slot
+template <int NP> struct TcSmem {
+  static constexpr int S = TcShape<NP>::S;
+  static constexpr uint32_t kStage = kTcAtile + NP * kTcK * 4;
   static constexpr uint32_t kBars = S * kStage;
-  static constexpr uint32_t kBytes = kBars + 8 * (2 * S + 1) + 8 + 1024;  // + alignment slack
+  static constexpr uint32_t kBytes = kBars + 8 * (3 * S + 5) + 16 + 1024;  // + alignment slack
 };
 
-// BS = 0: B's hi and lo parts arrive packed (two TMA loads a stage); BS = 1: the raw B arrives
-// (one load) and is split in shared memory like A
-template <int NP, int S, int BS = 0>
-__global__ void __launch_bounds__(kTcThreads, 1)
-    k_zgemm_tc(const __grid_constant__ CUtensorMap mbh, const __grid_constant__ CUtensorMap mbl,
-               const CUtensorMap* __restrict__ ma, const TcTile* __restrict__ tiles,
-               const TcObj* __restrict__ objs, float2* __restrict__ y, int64_t vstride, int R,
-               int* err) {
-  typedef TcSmem<NP, S> L;
-  constexpr uint32_t kTx = kTcAtile + (BS ? 1 : 2) * L::kBtile;  // bytes landing per stage
-  constexpr uint32_t kIdesc = tf32_idesc(kTcM, NP);
+// one row of a landed FP32 tile (128 bytes, its 16-byte vectors swizzled by the row) scaled and turned
+// in place into 32 FP16 hi parts and 32 lo parts
+__device__ __forceinline__ void tc_convert_row(uint8_t* tile, int row, float s) {
+  float4* a = reinterpret_cast<float4*>(tile + row * 128);
+  const int x = row & 7;
+  float4 v[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) v[c] = a[c ^ x];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float4 p = v[2 * j], q = v[2 * j + 1];
+    uint4 hi, lo;
+    tc_halves(p.x * s, p.y * s, &hi.x, &lo.x);
+    tc_halves(p.z * s, p.w * s, &hi.y, &lo.y);
+    tc_halves(q.x * s, q.y * s, &hi.z, &lo.z);
+    tc_halves(q.z * s, q.w * s, &hi.w, &lo.w);
+    reinterpret_cast<uint4*>(a)[j ^ x] = hi;
+    reinterpret_cast<uint4*>(a)[(4 + j) ^ x] = lo;
+  }
+}
+
+// Persistent CTAs, one per SM; CTA b takes the units b, b + gridDim.x, ... (nst[b] stages in all): a unit
+// is the stages [k0, k1) of the K loop of one 128-row tile of one block of one of the two matrices.
+// Warps 0-3 read the accumulators, warp 4 issues the TMA loads, warp 5 the MMAs, the others convert the
+// landed tiles; stages pass from one to the next through mbarriers and run on across units, and
+// (NP <= 128) the accumulators are double, so a unit's start-up and its epilogue cost nothing. A_hi
+// B_hi is accumulated apart from the cross terms (NP columns each): the tensor core truncates every
+// accumulation, and the cross terms, 2^-11 as large, would triple the number of truncations of the
+// large sum. The parts of a tile cut into several units go to a workspace, which k_tc_reduce sums (the
+// unit that finishes last, four warps on one SM, took 50 us for it).
+template <int NP>
+__global__ void __launch_bounds__(tc_threads<NP>(), 1)
+    k_zgemm_tc(const __grid_constant__ CUtensorMap mb, const CUtensorMap* __restrict__ mz,
+               const CUtensorMap* __restrict__ mc, const TcUnit* __restrict__ units, int nunit,
+               const int32_t* __restrict__ nst, const TcObj* __restrict__ objs,
+               const int32_t* __restrict__ shz, const int32_t* __restrict__ shc,
+               const int32_t* __restrict__ shb, float2* __restrict__ yz, float2* __restrict__ yc,
+               int64_t vstride, int R, float4* __restrict__ part, int* err) {
+  typedef TcSmem<NP> L;
+  constexpr int S = L::S, kG = TcShape<NP>::G;
+  constexpr int NACC = NP <= 128 ? 2 : 1;          // accumulator pairs in TMEM
+  constexpr uint32_t kCols = NACC * 2 * NP;
+  constexpr uint32_t kTx = L::kStage;              // bytes landing per stage
+  constexpr uint32_t kIdesc = f16_idesc(kTcM, NP);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(base + L::kBars);
-  uint64_t* empty = full + S;
-  uint64_t* done = empty + S;
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
+  uint64_t* full = reinterpret_cast<uint64_t*>(base + L::kBars);  // [S] the stage's loads have landed
+  uint64_t* conv = full + S;                                      // [S] its A tile is converted
+  uint64_t* empty = conv + S;                                     // [S] its MMAs are done
+  uint64_t* done = empty + S;                                     // [2] a unit's accumulators are final
+  uint64_t* taken = done + 2;                                     // [2] ... and have been read
+  uint64_t* fin = taken + 2;                                      // clean-up
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(fin + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const TcTile t = tiles[blockIdx.x];
-  const TcObj o = objs[t.obj];
-  const CUtensorMap* mA = ma + t.obj;
-  const int nk = (2 * o.n + kTcK - 1) / kTcK;
   int* const abort_flag = err + 1;  // set by any CTA of this launch that gave up
 
   // a CTA that starts after another one gave up leaves at once (one decision for the block)
-  __shared__ int s_skip;
-  if (tid == 0) s_skip = *(const volatile int*)abort_flag;
+  __shared__ int s_flag, s_fail;
+  if (tid == 0) {
+    s_flag = *(const volatile int*)abort_flag;
+    s_fail = 0;
+  }
   __syncthreads();
-  if (s_skip) return;
+  if (s_flag) return;
 
   if (tid == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 1);
+      mbar_init(&conv[s], kG / 32);
       mbar_init(&empty[s], 1);
     }
-    mbar_init(done, 1);
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&done[q], 1);
+      mbar_init(&taken[q], kTcEpi / 32);
+    }
+    mbar_init(fin, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) tc_alloc(tslot, NP);
+  if (warp == 5) tc_alloc(tslot, kCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = *tslot;  // pair q: columns 2 NP q + [0, NP) A_hi B_hi, + [NP, 2 NP) the cross terms
 
-  // thread 0's bookkeeping: chunks 0..issued-1 have their loads issued; no load after a failed wait
-  int issued = 0;
-  bool stalled = false;
-  auto load = [&](int kc) {
-    const int s = kc % S;
-    uint8_t* st = base + s * L::kStage;
-    const int kx = (int)(o.koff + (int64_t)kc * kTcK);
-    mbar_arrive_tx(&full[s], kTx);
-    tma_load_2d(st, mA, kc * kTcK, t.row0, &full[s]);
-    tma_load_2d(st + 2 * kTcAtile, &mbh, kx, 0, &full[s]);
-    if constexpr (BS == 0) tma_load_2d(st + 2 * kTcAtile + L::kBtile, &mbl, kx, 0, &full[s]);
-    issued = kc + 1;
-  };
-  if (tid == 0) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(mA)) : "memory");
-    for (int kc = 0; kc < nk && kc < S; ++kc) load(kc);
-  }
-
-  int kc_fail = -1;  // block-uniform: the chunk whose wait timed out for some thread
-  for (int kc = 0; kc < nk; ++kc) {
-    const int s = kc % S;
-    const bool ok = tc_wait(&full[s], (kc / S) & 1, abort_flag, kTcSpin);
-    if (ok) {  // split the A tile: hi in place, lo beside it (same offsets, same swizzle)
-      float4* a = reinterpret_cast<float4*>(base + s * L::kStage);
-      float4* al = reinterpret_cast<float4*>(base + s * L::kStage + kTcAtile);
-#pragma unroll 4
-      for (int i = tid; i < (int)(kTcAtile / 16); i += kTcThreads) {
-        const float4 v = a[i];
-        const float4 h = make_float4(tf32_hi(v.x), tf32_hi(v.y), tf32_hi(v.z), tf32_hi(v.w));
-        a[i] = h;
-        al[i] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
+  int issued = 0;  // producer: stages whose loads are issued
+  bool ok = true;
+  if (warp < 4) {
+    // accumulators out: thread = row of the tile; warp 0 decides for the four (they share barriers)
+    const int trow = tid;
+    int n = 0;
+    for (int ui = blockIdx.x; ui < nunit; ui += gridDim.x, ++n) {
+      const TcUnit u = units[ui];
+      const TcObj o = objs[u.obj];
+      const int q = n % NACC;
+      if (warp == 0) {
+        ok = __all_sync(0xffffffffu, tc_wait(&done[q], (n / NACC) & 1, abort_flag, kTcSpin));
+        if (lane == 0) s_flag = ok;
       }
-      if constexpr (BS == 1) {  // the same split of the raw B tile
-        float4* b = reinterpret_cast<float4*>(base + s * L::kStage + 2 * kTcAtile);
-        float4* bl = reinterpret_cast<float4*>(base + s * L::kStage + 2 * kTcAtile + L::kBtile);
-#pragma unroll 4
-        for (int i = tid; i < (int)(L::kBtile / 16); i += kTcThreads) {
-          const float4 v = b[i];
-          const float4 h = make_float4(tf32_hi(v.x), tf32_hi(v.y), tf32_hi(v.z), tf32_hi(v.w));
-          b[i] = h;
-          bl[i] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      if (!*(volatile int*)&s_flag) break;
+      tc_fence_after();
+      const int row = u.row0 + trow, cend = min(NP, (2 * R + 15) & ~15);
+      float2* y = u.mat ? yc : yz;
+      const int sa = row < o.n ? (u.mat ? shc : shz)[o.xoff + row] : 0;
+      const int32_t* sb = shb + u.obj * (int64_t)kTcMaxRhs;
+      const uint32_t tl = tmem + 2 * NP * q + ((uint32_t)(warp * 32) << 16);
+      for (int c0 = 0; c0 < cend; c0 += 16) {
+        float v[16], w[16];
+        tc_ld16(tl + c0, v);
+        tc_ld16(tl + NP + c0, w);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] += w[k];
+        if (u.parts > 1) {
+          float4* p = part + (int64_t)u.slot * (kTcM * NP / 4) + (c0 / 4) * kTcM + trow;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) p[k * kTcM] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+        } else if (row < o.n) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const int r = c0 / 2 + k;
+            if (r < R) y[r * vstride + o.xoff + row] = tc_unscale(v[2 * k], v[2 * k + 1], sa + __ldg(sb + r));
+          }
         }
       }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&taken[q]);
+      asm volatile("bar.sync 1, 128;" ::: "memory");  // s_flag is rewritten by the next unit
+    }
+  } else if (warp == 4) {
+    if (lane == 0) {
+      int slot = 0, ph = 1;  // ph: parity of the stage's previous MMAs (the first pass waits for none)
+      for (int ui = blockIdx.x; ui < nunit && ok; ui += gridDim.x) {
+        const TcUnit u = units[ui];
+        const TcObj o = objs[u.obj];
+        const CUtensorMap* mA = (u.mat ? mc : mz) + u.obj;
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(mA)) : "memory");
+        for (int kc = u.k0; kc < u.k1; ++kc) {
+          if (issued >= S && !tc_wait(&empty[slot], ph, abort_flag, kTcSpin)) {
+            ok = false;
+            break;
+          }
+          uint8_t* st = base + slot * L::kStage;
+          const int kx = (int)(o.koff + (int64_t)kc * kTcK);
+          mbar_arrive_tx(&full[slot], kTx);
+          tma_load_2d(st, mA, kc * kTcK, u.row0, &full[slot]);
+          tma_load_2d(st + kTcAtile, &mb, kx, 0, &full[slot]);
+          ++issued;
+          if (++slot == S) {
+            slot = 0;
+            ph ^= 1;
+          }
+        }
+      }
+    }
+  } else if (warp == 5) {
+    if (lane == 0) {
+      int slot = 0, ph = 0, n = 0;
+      for (int ui = blockIdx.x; ui < nunit && ok; ui += gridDim.x, ++n) {
+        const int k0 = units[ui].k0, k1 = units[ui].k1, q = n % NACC;
+        if (n >= NACC && !tc_wait(&taken[q], (n / NACC - 1) & 1, abort_flag, kTcSpin)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem + 2 * NP * q;
+        for (int kc = k0; kc < k1; ++kc) {
+          if (!tc_wait(&full[slot], ph, abort_flag, kTcSpin) || !tc_wait(&conv[slot], ph, abort_flag, kTcSpin)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sa = smem_u32(base + slot * L::kStage), sb = sa + kTcAtile;
+#pragma unroll
+          for (int k = 0; k < kTcK / 16; ++k) {  // 16 FP16 = 32 bytes of K per instruction; lo 64 bytes on
+            const uint64_t ah = sw128_desc(sa + 32 * k), al = sw128_desc(sa + 64 + 32 * k);
+            const uint64_t bh = sw128_desc(sb + 32 * k), bl = sw128_desc(sb + 64 + 32 * k);
+            const uint32_t acc = (kc > k0 || k > 0) ? 1u : 0u;
+            tc_mma_f16(d, ah, bh, kIdesc, acc);
+            tc_mma_f16(d + NP, al, bh, kIdesc, acc);
+            tc_mma_f16(d + NP, ah, bl, kIdesc, 1u);
+          }
+          tc_commit(&empty[slot]);
+          if (++slot == S) {
+            slot = 0;
+            ph ^= 1;
+          }
+        }
+        if (ok) tc_commit(&done[q]);
+      }
+    }
+  } else {
+    // a group converts the stages of its slot, a thread the rows t, t + kG, ... of each
+    constexpr int kRows = kTcM / kG;
+    const int t = (tid - 192) % kG, slot = (tid - 192) / kG, total = nst[blockIdx.x];
+    int ph = 0, ui = blockIdx.x, first = 0, last = 0;  // stages [first, last) belong to unit ui
+    float sc[kRows];
+    for (int i = slot; i < total; i += S, ph ^= 1) {
+      bool moved = last == 0;
+      if (moved) last = units[ui].k1 - units[ui].k0;
+      while (i >= last) {
+        ui += gridDim.x;
+        first = last;
+        last = first + units[ui].k1 - units[ui].k0;
+        moved = true;
+      }
+      if (moved) {
+        const TcUnit u = units[ui];
+        const TcObj o = objs[u.obj];
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) {
+          const int row = u.row0 + t + k * kG;
+          sc[k] = row < o.n ? tc_pow2((u.mat ? shc : shz)[o.xoff + row]) : 0.f;
+        }
+      }
+      ok = tc_wait(&full[slot], ph, abort_flag, kTcSpin);
+      if (!__all_sync(0xffffffffu, ok)) {
+        ok = false;
+        break;
+      }
+      uint8_t* st = base + slot * L::kStage;
+#pragma unroll
+      for (int k = 0; k < kRows; ++k) tc_convert_row(st, t + k * kG, sc[k]);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    }
-    if (__syncthreads_or(!ok)) {
-      kc_fail = kc;
-      break;
-    }
-    if (tid == 0) {
-      tc_fence_after();
-      const uint32_t sa = smem_u32(base + s * L::kStage);
-      const uint32_t sb = sa + 2 * kTcAtile;
-#pragma unroll
-      for (int k = 0; k < kTcK / 8; ++k) {  // 8 TF32 = 32 bytes of K per instruction
-        const uint64_t ah = sw128_desc(sa + 32 * k), alo = sw128_desc(sa + kTcAtile + 32 * k);
-        const uint64_t bh = sw128_desc(sb + 32 * k), blo = sw128_desc(sb + L::kBtile + 32 * k);
-        tc_mma_tf32(tmem, alo, bh, kIdesc, (kc > 0 || k > 0) ? 1u : 0u);
-        tc_mma_tf32(tmem, ah, blo, kIdesc, 1u);
-        tc_mma_tf32(tmem, ah, bh, kIdesc, 1u);
-      }
-      tc_commit(&empty[s]);
-      // the previous chunk's stage takes chunk kc - 1 + S once that chunk's MMAs are done
-      const int nxt = kc - 1 + S;
-      if (kc >= 1 && nxt < nk && !stalled) {
-        if (tc_wait(&empty[(kc - 1) % S], ((kc - 1) / S) & 1, abort_flag, kTcSpin)) load(nxt);
-        else stalled = true;  // the loop's next wait on chunk nxt times out for every thread
-      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&conv[slot]);
     }
   }
-
-  bool ok = kc_fail < 0;
-  if (ok) {
-    if (tid == 0) tc_commit(done);
-    ok = !__syncthreads_or(!tc_wait(done, 0, abort_flag, kTcSpin));
-    if (!ok) kc_fail = nk;
+  if (!ok) {
+    s_fail = 1;
+    atomicExch(err, 1);
+    atomicExch(abort_flag, 1);
   }
-  if (!ok) {  // leave cleanly: error code, MMAs and copies in flight waited for (bounded)
-    if (tid == 0) {
-      atomicExch(err, 1);
-      atomicExch(abort_flag, 1);
-      if (kc_fail < nk) tc_commit(done);
-      const int none = 0;  // the cleanup waits run their own short limit to the end
-      tc_wait(done, 0, &none, kTcSpinCleanup);
-      for (int c = max(kc_fail, 0); c < issued; ++c) tc_wait(&full[c % S], (c / S) & 1, &none, kTcSpinCleanup);
+  __syncwarp();
+  __syncthreads();
+  if (s_fail) {  // leave cleanly: MMAs and copies in flight waited for (bounded)
+    const int none = 0;  // these waits run their own short limit to the end
+    if (warp == 5 && lane == 0) {
+      tc_commit(fin);
+      tc_wait(fin, 0, &none, kTcSpinCleanup);
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (warp == 0) tc_dealloc(tmem, NP);
-    return;
-  }
-
-  tc_fence_after();
-  const int row = t.row0 + warp * 32 + lane;
-  const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
-  for (int c0 = 0; c0 < 2 * R && c0 < NP; c0 += 16) {
-    float v[16];
-    tc_ld16(tl + c0, v);
-    if (row < o.n) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int r = c0 / 2 + q;
-        if (r < R) y[r * vstride + o.xoff + row] = make_float2(v[2 * q], v[2 * q + 1]);
-      }
-    }
+    if (warp == 4 && lane == 0)
+      for (int c = max(issued - S, 0); c < issued; ++c) tc_wait(&full[c % S], (c / S) & 1, &none, kTcSpinCleanup);
+    __syncwarp();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 0) tc_dealloc(tmem, NP);
+  if (warp == 5) tc_dealloc(tmem, kCols);
+}
+
+// y of the tiles cut along K: the sum of their parts in order; one CTA per tile and 16 columns
+template <int NP>
+__global__ void __launch_bounds__(kTcM) k_tc_reduce(const TcUnit* __restrict__ tiles, const TcObj* __restrict__ objs,
+                                                    const int32_t* __restrict__ shz, const int32_t* __restrict__ shc,
+                                                    const int32_t* __restrict__ shb, const float4* __restrict__ part,
+                                                    float2* __restrict__ yz, float2* __restrict__ yc,
+                                                    int64_t vstride, int R) {
+  const TcUnit u = tiles[blockIdx.x];
+  const TcObj o = objs[u.obj];
+  const int row = u.row0 + threadIdx.x, c0 = 16 * blockIdx.y;
+  if (row >= o.n) return;
+  const float4* p = part + (int64_t)u.slot0 * (kTcM * NP / 4) + (c0 / 4) * kTcM + threadIdx.x;
+  float4 a[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) a[c] = p[c * kTcM];
+#pragma unroll 4
+  for (int k = 1; k < u.parts; ++k) {
+    p += kTcM * NP / 4;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float4 t = p[c * kTcM];
+      a[c] = make_float4(a[c].x + t.x, a[c].y + t.y, a[c].z + t.z, a[c].w + t.w);
+    }
+  }
+  const int sa = (u.mat ? shc : shz)[o.xoff + row];
+  const int32_t* sb = shb + u.obj * (int64_t)kTcMaxRhs;
+  float2* y = (u.mat ? yc : yz) + o.xoff + row;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int r = c0 / 2 + 2 * c;
+    if (r < R) y[r * vstride] = tc_unscale(a[c].x, a[c].y, sa + __ldg(sb + r));
+    if (r + 1 < R) y[(r + 1) * vstride] = tc_unscale(a[c].z, a[c].w, sa + __ldg(sb + r + 1));
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -345,18 +539,27 @@ typedef PFN_cuTensorMapEncodeTiled_v12000 TcEncode;
 struct TcState {
   CUtensorMap* mz = nullptr;  // per object, over the FP32 Z and C blocks (device)
   CUtensorMap* mc = nullptr;
-  TcTile* tiles = nullptr;
-  int ntiles = 0;
+  struct Units {
+    TcUnit* d = nullptr;
+    int32_t* nst = nullptr;   // [ctas] stages of each persistent CTA
+    TcUnit* cut = nullptr;    // [ncut] first unit of every tile cut along K
+    int n = 0, ncut = 0, slots = 0, ctas = 0;
+  } units[3];                 // Z alone, C alone, both
   TcObj* objs = nullptr;
-  int32_t* slot = nullptr;    // [nslot] unknown of each padded slot, -1 in padding
-  int64_t nslot = 0;          // sum of ld_i
-  float *bh = nullptr, *bl = nullptr;  // packed B, [np_cap][2 nslot] each
+  int64_t ktot = 0;           // 32-bit words per row of the packed B
+  uint32_t* b = nullptr;      // packed B, [np_cap][ktot]
+  int32_t *shz = nullptr, *shc = nullptr;  // [ne] exponent shifts of the rows of Z and C
+  int32_t* shb = nullptr;     // [nobj][kTcMaxRhs] of the right-hand sides' slices
+  float4* part = nullptr;     // partial sums of tiles cut along K
   int np_cap = 0;
   int* err = nullptr;         // [2]: a wait timed out in some product (sticky); this launch gave up
   int64_t calls = 0;
   ~TcState() {
-    for (void* p : {(void*)mz, (void*)mc, (void*)tiles, (void*)objs, (void*)slot, (void*)bh,
-                    (void*)bl, (void*)err})
+    for (Units& u : units)
+      for (void* p : {(void*)u.d, (void*)u.nst, (void*)u.cut})
+        if (p) cudaFree(p);
+    for (void* p : {(void*)mz, (void*)mc, (void*)objs, (void*)b, (void*)shz, (void*)shc, (void*)shb, (void*)part,
+                    (void*)err})
       if (p) cudaFree(p);
   }
 };
@@ -396,7 +599,59 @@ static int tc_map(TcEncode enc, CUtensorMap* m, const void* base, int64_t inner,
   return BEM_OK;
 }
 
-// tiles, object table, slot table and the per-object tensor maps of Z and C (first use)
+// The units of a product over the matrices in `mats` (bit 0 Z, bit 1 C): every tile's K loop is cut
+// into equal parts of at most Lmax stages, Lmax the shortest for which there are at most w units per
+// SM; w is the one with the least w Lmax, plus kTcOver where that cuts any tile (the stages that the
+// trip through the workspace costs, about 6 us). Longest first, dealt to the CTAs in turn.
+constexpr int kTcOver = 12, kTcMaxParts = 16;
+static std::vector<TcUnit> tc_units(const std::vector<TcObj>& objs, int mats, int nsm, int* slots) {
+  struct T { int obj, row0, mat, nk; };
+  std::vector<T> ts;
+  int longest = 0;
+  for (int m = 0; m < 2; ++m)
+    if (mats >> m & 1)
+      for (int i = 0; i < (int)objs.size(); ++i)
+        for (int r0 = 0; r0 < objs[i].n; r0 += kTcM) {
+          ts.push_back({i, r0, m, (2 * objs[i].n + kTcK - 1) / kTcK});
+          longest = std::max(longest, ts.back().nk);
+        }
+  auto count = [&](int L) {
+    int64_t c = 0;
+    for (const T& t : ts) c += (t.nk + L - 1) / L;
+    return c;
+  };
+  const int shortest = std::max(1, (longest + kTcMaxParts - 1) / kTcMaxParts);
+  int best = longest;
+  int64_t cost = INT64_MAX;
+  for (int w = 1; w <= 8; ++w) {
+    int lo = shortest, hi = longest;  // smallest L with count(L) <= w nsm
+    if (count(hi) > (int64_t)w * nsm) continue;
+    while (lo < hi) {
+      const int mid = (lo + hi) / 2;
+      if (count(mid) <= (int64_t)w * nsm) hi = mid;
+      else lo = mid + 1;
+    }
+    const int64_t c = (int64_t)w * lo + (lo < longest ? kTcOver : 0);
+    if (c < cost) {
+      cost = c;
+      best = lo;
+    }
+  }
+  std::vector<TcUnit> us;
+  *slots = 0;
+  for (int i = 0; i < (int)ts.size(); ++i) {
+    const T& t = ts[i];
+    const int p = (t.nk + best - 1) / best, s0 = *slots;
+    for (int q = 0; q < p; ++q)
+      us.push_back(TcUnit{t.obj, t.row0, t.mat, (int)((int64_t)t.nk * q / p), (int)((int64_t)t.nk * (q + 1) / p),
+                          p, s0 + q, s0});
+    if (p > 1) *slots += p;
+  }
+  std::stable_sort(us.begin(), us.end(), [](const TcUnit& a, const TcUnit& b) { return a.k1 - a.k0 > b.k1 - b.k0; });
+  return us;
+}
+
+// units, object table, slot table and the per-object tensor maps of Z and C (first use)
 static int tc_prepare(aim_ctx* c, TcState** out) {
   if (c->tc) {
     *out = static_cast<TcState*>(c->tc);
@@ -413,29 +668,22 @@ static int tc_prepare(aim_ctx* c, TcState** out) {
   }
   TcState* t = new TcState();
   std::vector<TcObj> objs(c->nobj);
-  std::vector<TcTile> tiles;
-  std::vector<int32_t> slot;
+  int64_t ktot = 0;
   std::vector<CUtensorMap> mz(c->nobj), mc(c->nobj);
   int rc = BEM_OK;
   for (int i = 0, xo = 0; i < c->nobj && rc == BEM_OK; ++i) {
     const int n = c->e1[i] - c->e0[i], ld = c->zld[i];
-    objs[i] = TcObj{n, xo, 2 * (int64_t)slot.size()};
-    for (int l = 0; l < ld; ++l) slot.push_back(l < n ? xo + l : -1);
-    for (int r0 = 0; r0 < n; r0 += kTcM) tiles.push_back(TcTile{i, r0});
+    objs[i] = TcObj{n, xo, ktot};
+    ktot += 2 * round_up(n, 16);
     rc = tc_map(enc, &mz[i], c->f32.Z + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcM);
     if (rc == BEM_OK) rc = tc_map(enc, &mc[i], c->f32.C + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcM);
     xo += n;
   }
-  if (rc == BEM_OK && 2 * (int64_t)slot.size() > INT32_MAX) {
+  if (rc == BEM_OK && ktot > INT32_MAX) {
     set_error("tensor-core product: more than 2^30 unknowns");
     rc = BEM_EINVAL;
   }
-  // largest blocks first: their tiles carry the longest K loops
-  std::stable_sort(tiles.begin(), tiles.end(), [&](const TcTile& a, const TcTile& b) {
-    return objs[a.obj].n > objs[b.obj].n;
-  });
-  t->ntiles = (int)tiles.size();
-  t->nslot = (int64_t)slot.size();
+  t->ktot = ktot;
   auto up = [&](void** p, const void* h, size_t bytes) {
     if (rc != BEM_OK) return;
     if (cudaMalloc(p, bytes) != cudaSuccess || cudaMemcpy(*p, h, bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -445,11 +693,48 @@ static int tc_prepare(aim_ctx* c, TcState** out) {
   };
   up((void**)&t->mz, mz.data(), mz.size() * sizeof(CUtensorMap));
   up((void**)&t->mc, mc.data(), mc.size() * sizeof(CUtensorMap));
-  up((void**)&t->tiles, tiles.data(), tiles.size() * sizeof(TcTile));
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  for (int m = 0; m < 3; ++m) {
+    TcState::Units& q = t->units[m];
+    const std::vector<TcUnit> us = tc_units(objs, m == 2 ? 3 : m + 1, std::max(nsm, 1), &q.slots);
+    q.n = (int)us.size();
+    q.ctas = std::min(q.n, std::max(nsm, 1));
+    std::vector<int32_t> nst(q.ctas, 0);
+    for (int i = 0; i < q.n; ++i) nst[i % q.ctas] += us[i].k1 - us[i].k0;
+    up((void**)&q.nst, nst.data(), nst.size() * sizeof(int32_t));
+    std::vector<TcUnit> cut;
+    for (const TcUnit& v : us)
+      if (v.parts > 1 && v.slot == v.slot0) cut.push_back(v);
+    q.ncut = (int)cut.size();
+    if (q.ncut > 0) up((void**)&q.cut, cut.data(), cut.size() * sizeof(TcUnit));
+    up((void**)&q.d, us.data(), us.size() * sizeof(TcUnit));
+  }
   up((void**)&t->objs, objs.data(), objs.size() * sizeof(TcObj));
-  up((void**)&t->slot, slot.data(), slot.size() * sizeof(int32_t));
   const int zero[2] = {0, 0};  // [0]: a wait timed out in some product; [1]: this launch gave up
   up((void**)&t->err, zero, sizeof(zero));
+  // exponent shifts of the matrices' rows
+  int64_t* doff = nullptr;
+  int nmax = 0;
+  for (const TcObj& o : objs) nmax = std::max(nmax, o.n);
+  const std::vector<int32_t> none((size_t)std::max<int64_t>(c->ne, c->nobj * (int64_t)kTcMaxRhs), 0);
+  up((void**)&t->shz, none.data(), (size_t)c->ne * sizeof(int32_t));
+  up((void**)&t->shc, none.data(), (size_t)c->ne * sizeof(int32_t));
+  up((void**)&t->shb, none.data(), (size_t)c->nobj * kTcMaxRhs * sizeof(int32_t));
+  up((void**)&doff, c->zoff.data(), (size_t)c->nobj * sizeof(int64_t));
+  if (rc == BEM_OK && nmax > 0) {
+    for (int o0 = 0; o0 < c->nobj; o0 += 65535) {  // gridDim.y
+      const dim3 g((nmax + 7) / 8, std::min(65535, c->nobj - o0));
+      k_tc_rowshift<<<g, 256>>>(t->objs + o0, doff + o0, c->f32.Z, t->shz);
+      k_tc_rowshift<<<g, 256>>>(t->objs + o0, doff + o0, c->f32.C, t->shc);
+    }
+    if (cudaDeviceSynchronize() != cudaSuccess) {
+      set_error("tensor-core product: %s", cudaGetErrorString(cudaGetLastError()));
+      rc = BEM_ECUDA;
+    }
+  }
+  if (doff) cudaFree(doff);
   if (rc != BEM_OK) {
     delete t;
     return rc;
@@ -459,16 +744,20 @@ static int tc_prepare(aim_ctx* c, TcState** out) {
   return BEM_OK;
 }
 
-template <int NP, int S, int BS>
-static int tc_launch(TcState* t, const CUtensorMap& mbh, const CUtensorMap& mbl, const CUtensorMap* ma,
-                     float2* y, int64_t vstride, int R, cudaStream_t s) {
-  constexpr uint32_t kSmem = TcSmem<NP, S>::kBytes;
+template <int NP>
+static int tc_launch(TcState* t, const CUtensorMap& mb, float2* yz, float2* yc, int64_t vstride, int R,
+                     cudaStream_t s) {
+  constexpr uint32_t kSmem = TcSmem<NP>::kBytes;
   static_assert(kSmem <= 227 * 1024, "shared memory per CTA");
+  const TcState::Units& q = t->units[yz && yc ? 2 : yz ? 0 : 1];
   // per call: the attribute belongs to the current device (cheap next to the product)
-  BEM_CUDA(cudaFuncSetAttribute(k_zgemm_tc<NP, S, BS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
+  BEM_CUDA(cudaFuncSetAttribute(k_zgemm_tc<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
   BEM_CUDA(cudaMemsetAsync(t->err + 1, 0, sizeof(int), s));
-  k_zgemm_tc<NP, S, BS><<<t->ntiles, kTcThreads, kSmem, s>>>(mbh, mbl, ma, t->tiles, t->objs, y, vstride,
-                                                            R, t->err);
+  k_zgemm_tc<NP><<<q.ctas, tc_threads<NP>(), kSmem, s>>>(mb, t->mz, t->mc, q.d, q.n, q.nst, t->objs, t->shz,
+                                                         t->shc, t->shb, yz, yc, vstride, R, t->part, t->err);
+  if (q.ncut > 0)
+    k_tc_reduce<NP><<<dim3(q.ncut, (2 * R + 15) / 16), kTcM, 0, s>>>(q.cut, t->objs, t->shz, t->shc, t->shb, t->part,
+                                                                     yz, yc, vstride, R);
   BEM_CUDA(cudaGetLastError());
   return BEM_OK;
 }
@@ -477,7 +766,7 @@ static int tc_launch(TcState* t, const CUtensorMap& mbh, const CUtensorMap& mbl,
 int internal_tc(aim_ctx* c, const float2* h, float2* e, float2* heq, int nrhs, cudaStream_t s) {
   TcState* t = nullptr;
   BEM_TRY(tc_prepare(c, &t));
-  if (t->ntiles == 0) return BEM_OK;
+  if (t->units[0].n == 0) return BEM_OK;
   TcEncode enc = tc_encoder();
   const int64_t ne = c->ne;
   for (int r0 = 0; r0 < nrhs; r0 += kTcMaxRhs) {
@@ -485,41 +774,35 @@ int internal_tc(aim_ctx* c, const float2* h, float2* e, float2* heq, int nrhs, c
     const int NP = R <= 16 ? 32 : R <= 32 ? 64 : R <= 64 ? 128 : 256;
     if (NP > t->np_cap) {
       BEM_CUDA(cudaStreamSynchronize(s));  // the old workspace may be in use on s
-      if (t->bh) cudaFree(t->bh);
-      if (t->bl) cudaFree(t->bl);
-      t->bh = t->bl = nullptr;
+      if (t->b) cudaFree(t->b);
+      if (t->part) cudaFree(t->part);
+      t->b = nullptr;
+      t->part = nullptr;
       t->np_cap = 0;
-      const size_t bytes = (size_t)NP * 2 * t->nslot * sizeof(float);
-      if (cudaMalloc((void**)&t->bh, bytes) != cudaSuccess || cudaMalloc((void**)&t->bl, bytes) != cudaSuccess) {
+      const size_t bytes = (size_t)NP * t->ktot * sizeof(uint32_t);
+      int slots = 0;
+      for (const TcState::Units& q : t->units) slots = std::max(slots, q.slots);
+      const size_t pbytes = (size_t)slots * kTcM * NP * sizeof(float) + 16;
+      if (cudaMalloc((void**)&t->b, bytes) != cudaSuccess || cudaMalloc((void**)&t->part, pbytes) != cudaSuccess) {
         set_error("tensor-core product: no device memory for the packed right-hand sides");
         return BEM_ENOMEM;
       }
       t->np_cap = NP;
     }
-    // form 1 packs the raw values only (B split in shared memory); the second map is then unused
-    const bool raw = c->tc_variant == 1;
-    CUtensorMap mbh, mbl;
-    BEM_TRY(tc_map(enc, &mbh, t->bh, 2 * t->nslot, NP, 2 * t->nslot * (int64_t)sizeof(float), NP));
-    BEM_TRY(tc_map(enc, &mbl, t->bl, 2 * t->nslot, NP, 2 * t->nslot * (int64_t)sizeof(float), NP));
-    const dim3 pg((unsigned)((t->nslot + 255) / 256), NP / 2);
-    k_tc_pack<<<pg, 256, 0, s>>>(h + r0 * ne, ne, R, t->slot, t->nslot, t->bh, raw ? nullptr : t->bl);
+    CUtensorMap mb;  // 32 words of a row are one stage
+    BEM_TRY(tc_map(enc, &mb, t->b, t->ktot, NP, t->ktot * (int64_t)sizeof(uint32_t), NP));
+    k_tc_pack<<<dim3(c->nobj, NP / 2), 256, 0, s>>>(h + r0 * ne, ne, R, t->objs, t->ktot, t->b, t->shb);
     BEM_CUDA(cudaGetLastError());
-    for (int w = 0; w < 2; ++w) {
-      float2* y = w == 0 ? e : heq;
-      if (!y) continue;
-      const CUtensorMap* ma = w == 0 ? t->mz : t->mc;
-      y += r0 * ne;
-#define BEM_TC(NPV, SV)                                                               \
-  BEM_TRY(raw ? (tc_launch<NPV, SV, 1>(t, mbh, mbl, ma, y, ne, R, s))                 \
-              : (tc_launch<NPV, SV, 0>(t, mbh, mbl, ma, y, ne, R, s)))
-      switch (NP) {
-        case 32: BEM_TC(32, 5); break;
-        case 64: BEM_TC(64, 4); break;
-        case 128: BEM_TC(128, 3); break;
-        default: BEM_TC(256, 2); break;
-      }
-#undef BEM_TC
+    float2* yz = e ? e + r0 * ne : nullptr;
+    float2* yc = heq ? heq + r0 * ne : nullptr;
+#define BEM_TC(NPV) BEM_TRY(tc_launch<NPV>(t, mb, yz, yc, ne, R, s))
+    switch (NP) {
+      case 32: BEM_TC(32); break;
+      case 64: BEM_TC(64); break;
+      case 128: BEM_TC(128); break;
+      default: BEM_TC(256); break;
     }
+#undef BEM_TC
   }
   ++t->calls;
   return BEM_OK;
