@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libbem_aim.so")
 BUILD = os.path.join(HERE, "_build")
-SOURCES = ["api.cu", "geom.cpp", "sched.cpp", "setup.cu", "fft.cu", "hot.cu", "gmres.cu",
+SOURCES = ["api.cu", "geom.cpp", "sched.cpp", "setup.cu", "fft.cu", "fft_two.cu", "hot.cu", "gmres.cu",
            "noalloc.cu", "learned.cu", "gemv_tma.cu", "post.cu", "zsparse.cu",
            "zgemm_tc.cu", "layered.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

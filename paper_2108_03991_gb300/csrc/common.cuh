@@ -109,6 +109,7 @@ template <typename R> struct PrecBuf {
   V* Gz = nullptr;     // FP32: Ghat per z line [Py][Px][M][L] in the register z pass's lane order
   V* Gs = nullptr;     // FP32, slab passes: Ghat octant as [fx][fz][fy]
   V* tw[3] = {nullptr, nullptr, nullptr};  // twiddle tables of the three axes
+  V* tt[3] = {nullptr, nullptr, nullptr};  // FP32: those of the two-pass transforms (fft_two.cu)
   R* ix = nullptr;     // [ne][4] I_x values
   R* fdE = nullptr;    // [ne][2] (l/A+, l/A-) : (F D)^T rows
   R* fdT = nullptr;    // [nt][3] signed l/A for the triangle's edges : F D rows
@@ -416,6 +417,11 @@ int fft_conv(aim_ctx* c, PrecBuf<R>& b, const typename C2<R>::T* sigma, typename
              int ncomp, typename C2<R>::T* ws, cudaStream_t s);
 template <typename R> int make_twiddles(aim_ctx* c, PrecBuf<R>& b);
 int make_ghat(aim_ctx* c);
+// FP32 convolution by two-pass transforms (fft_two.cu): whether it has the grid's lengths, its tables,
+// the convolution
+bool two_path(const aim_ctx* c);
+int two_twiddles(aim_ctx* c);
+int two_conv(aim_ctx* c, const float2* sigma, float2* phi, int ncomp, float2* ws, cudaStream_t s);
 int rhs_plane_wave(aim_ctx* c, const double* pol, const double* kh, void* b, int prec,
                    cudaStream_t st);
 // builds (or rebuilds in another precision) the block-diagonal preconditioner; prec: BEM_C32

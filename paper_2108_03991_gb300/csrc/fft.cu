@@ -20,6 +20,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "fft_radix.cuh"
 
 namespace bem {
 
@@ -73,79 +74,6 @@ int smooth_length(int need) {
       while (n % r == 0) n /= r;
     if (n == 1) return m;
   }
-}
-
-// ---------------------------------------------------------------------------------------
-// butterflies (forward: exp(-2 pi i / R); inverse: conjugate)
-// ---------------------------------------------------------------------------------------
-template <typename V> __device__ __forceinline__ V mul_mi(V a, bool inv) {  // * (-i) or * (+i)
-  return inv ? mk(-a.y, a.x) : mk(a.y, -a.x);
-}
-
-template <typename V> __device__ __forceinline__ void bfly2(V* v) {
-  V a = v[0], b = v[1];
-  v[0] = cadd(a, b);
-  v[1] = csub(a, b);
-}
-
-template <typename V> __device__ __forceinline__ void bfly3(V* v, bool inv) {
-  typedef decltype(v[0].x) R;
-  const R h = (R)0.86602540378443864676;  // sin(2 pi / 3)
-  V t1 = cadd(v[1], v[2]);
-  V d = csub(v[1], v[2]);
-  V t2 = mul_mi(mk(h * d.x, h * d.y), inv);
-  V m = mk(v[0].x - (R)0.5 * t1.x, v[0].y - (R)0.5 * t1.y);
-  v[0] = cadd(v[0], t1);
-  v[1] = cadd(m, t2);
-  v[2] = csub(m, t2);
-}
-
-template <typename V> __device__ __forceinline__ void bfly4(V* v, bool inv) {
-  V y0 = cadd(v[0], v[2]), y1 = csub(v[0], v[2]), y2 = cadd(v[1], v[3]);
-  V y3 = mul_mi(csub(v[1], v[3]), inv);
-  v[0] = cadd(y0, y2);
-  v[1] = cadd(y1, y3);
-  v[2] = csub(y0, y2);
-  v[3] = csub(y1, y3);
-}
-
-template <typename V> __device__ __forceinline__ void bfly5(V* v, bool inv) {
-  typedef decltype(v[0].x) R;
-  const R c1 = (R)0.30901699437494742410, c2 = (R)-0.80901699437494742410;  // cos 2pi/5, 4pi/5
-  const R s1 = (R)0.95105651629515357212, s2 = (R)0.58778525229247312917;   // sin 2pi/5, 4pi/5
-  V t1 = cadd(v[1], v[4]), t2 = cadd(v[2], v[3]), t3 = csub(v[1], v[4]), t4 = csub(v[2], v[3]);
-  V a1 = mk(v[0].x + c1 * t1.x + c2 * t2.x, v[0].y + c1 * t1.y + c2 * t2.y);
-  V a2 = mk(v[0].x + c2 * t1.x + c1 * t2.x, v[0].y + c2 * t1.y + c1 * t2.y);
-  V b1 = mk(s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y);
-  V b2 = mk(s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y);
-  V ib1 = mul_mi(b1, inv), ib2 = mul_mi(b2, inv);  // (-i) b forward
-  v[0] = cadd(v[0], cadd(t1, t2));
-  v[1] = cadd(a1, ib1);
-  v[4] = csub(a1, ib1);
-  v[2] = cadd(a2, ib2);
-  v[3] = csub(a2, ib2);
-}
-
-template <typename V> __device__ __forceinline__ void bfly8(V* v, bool inv) {
-  typedef decltype(v[0].x) R;
-  const R r2 = (R)0.70710678118654752440;
-  V e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
-  bfly4(e, inv);
-  bfly4(o, inv);
-  // w8^k o[k]: w8 = exp(-i pi/4) forward
-  V w1 = inv ? mk(r2 * (o[1].x - o[1].y), r2 * (o[1].x + o[1].y))
-             : mk(r2 * (o[1].x + o[1].y), r2 * (o[1].y - o[1].x));
-  V w2 = mul_mi(o[2], inv);
-  V w3 = inv ? mk(-r2 * (o[3].x + o[3].y), r2 * (o[3].x - o[3].y))
-             : mk(r2 * (o[3].y - o[3].x), -r2 * (o[3].x + o[3].y));
-  v[0] = cadd(e[0], o[0]);
-  v[4] = csub(e[0], o[0]);
-  v[1] = cadd(e[1], w1);
-  v[5] = csub(e[1], w1);
-  v[2] = cadd(e[2], w2);
-  v[6] = csub(e[2], w2);
-  v[3] = cadd(e[3], w3);
-  v[7] = csub(e[3], w3);
 }
 
 __device__ __forceinline__ int sw(int e) { return e + (e >> 4); }  // shared-memory swizzle
@@ -888,8 +816,8 @@ template <typename V> static size_t plane_smem(int Px, int Py) {
 }
 
 // ---------------------------------------------------------------------------------------
-// slab passes (FP32, padded x-y planes too large for shared memory; the split-ring array's
-// 1024 x 1024 planes): three passes over a workspace X[c][kx][z][y] that holds, per component,
+// slab passes (FP32, padded x-y planes too large for shared memory whose lengths fft_two.cu does not
+// have: no two radices up to 32, 972 and 1000 the smallest): three passes over a workspace X[c][kx][z][y] that holds, per component,
 // the x-transformed data rows only (Px * nz * ny values):
 //   x forward : RY rows of one data plane per CTA, zero-padded to Px, FFT along x, stored
 //               kx-major so that pass two reads one contiguous nz x ny slab per kx
@@ -1040,190 +968,6 @@ __global__ void __launch_bounds__(256) k_slab_xinv(const float2* __restrict__ ws
   }
 }
 
-// Warp-line forms of the three slab passes, for planes whose x and y lengths are 32 M points
-// (M = 16 or 32): one warp holds one line, point n = lane + 32 n1 in register n1, and
-// transforms it in registers (the M-point DFTs, the twiddles W_P^(lane k1) read from the table,
-// five xor-shuffle stages across the lanes), leaving X[k1 + M bitrev(lane)] in register k1; the
-// inverse takes that order back. No Stockham passes through shared memory: the x passes keep
-// every value in registers, the y-z pass meets the nz lines of one kx in one shared buffer for
-// the z transforms.
-template <int M>
-__device__ __forceinline__ void wline_fwd(float2* v, const float2* __restrict__ tw, int lane) {
-  constexpr int P = 32 * M;
-  dft_reg<float2, M>(v, tw, P / M, false);
-#pragma unroll
-  for (int k1 = 1; k1 < M; ++k1) v[k1] = cmul(v[k1], __ldg(&tw[lane * k1]));
-#pragma unroll
-  for (int st = 0; st < 5; ++st) {
-    const int sp = 32 >> (st + 1);
-    const bool top = (lane & sp) == 0;
-    const float sg = top ? 1.f : -1.f;
-    const float2 we = top ? make_float2(1.f, 0.f) : __ldg(&tw[(lane & (sp - 1)) * (M << st)]);
-#pragma unroll
-    for (int k1 = 0; k1 < M; ++k1) {
-      const float2 p = shfl_x(v[k1], sp);
-      v[k1] = cmul(make_float2(sg * v[k1].x + p.x, sg * v[k1].y + p.y), we);
-    }
-  }
-}
-
-template <int M>
-__device__ __forceinline__ void wline_inv(float2* v, const float2* __restrict__ tw, int lane) {
-  constexpr int P = 32 * M;
-#pragma unroll
-  for (int st = 4; st >= 0; --st) {
-    const int sp = 32 >> (st + 1);
-    const bool top = (lane & sp) == 0;
-    const float sg = top ? 1.f : -1.f;
-    float2 we = make_float2(1.f, 0.f);
-    if (!top) {
-      we = __ldg(&tw[(lane & (sp - 1)) * (M << st)]);
-      we.y = -we.y;
-    }
-#pragma unroll
-    for (int k1 = 0; k1 < M; ++k1) {
-      const float2 own = cmul(v[k1], we);
-      const float2 p = shfl_x(own, sp);
-      v[k1] = make_float2(sg * own.x + p.x, sg * own.y + p.y);
-    }
-  }
-#pragma unroll
-  for (int k1 = 1; k1 < M; ++k1) {
-    float2 w = __ldg(&tw[lane * k1]);
-    w.y = -w.y;
-    v[k1] = cmul(v[k1], w);
-  }
-  dft_reg<float2, M>(v, tw, P / M, true);
-}
-
-// x forward: warp w takes row y0 + w of data plane z; its Px spectrum values meet the other
-// seven rows' in a shared tile [row][kx] (every 32nd entry skipped: two lanes per bank at most)
-// and leave as X[c][kx][z][y0 .. y0 + 7], 64-byte runs, instead of one 8-byte value per kx
-template <int M>
-__global__ void __launch_bounds__(256) k_wslab_xfwd(const float2* __restrict__ sigma,
-                                                    float2* __restrict__ ws,
-                                                    const float2* __restrict__ twx, SlabArgs a) {
-  extern __shared__ float2 tile[];  // [8 rows][TS]
-  constexpr int P = 32 * M, TS = P + P / 32 + 1;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int y0 = blockIdx.x * 8, y = y0 + warp, z = blockIdx.y, c = blockIdx.z;
-  if (y < a.ny) {  // warp-uniform
-    const float2* src = sigma + c * a.ng + ((int64_t)z * a.ny + y) * a.nx;
-    float2 v[M];
-#pragma unroll
-    for (int n1 = 0; n1 < M; ++n1) {
-      const int x = lane + 32 * n1;
-      v[n1] = x < a.nx ? src[x] : make_float2(0.f, 0.f);
-    }
-    wline_fwd<M>(v, twx, lane);
-    const int k2 = brev_l<32>(lane);
-#pragma unroll
-    for (int k1 = 0; k1 < M; ++k1) {
-      const int kx = k1 + M * k2;
-      tile[warp * TS + kx + (kx >> 5)] = v[k1];
-    }
-  }
-  __syncthreads();
-  const int nr = min(8, a.ny - y0);
-  float2* dst = ws + c * a.P3 + (int64_t)z * a.ny + y0;
-  for (int i = threadIdx.x; i < 8 * P; i += blockDim.x) {
-    const int kx = i >> 3, r = i & 7;
-    if (r < nr) dst[(int64_t)kx * a.nz * a.ny + r] = tile[r * TS + kx + (kx >> 5)];
-  }
-}
-
-// y-z fused for one kx: warp z transforms its y line, the nz lines meet in shared memory
-// (position k1 * 32 + lane) for the z DFTs and Ghat, then each warp inverts its line. Ghat is
-// read where it is used (each value serves the two positions ky and P - ky of this CTA, the
-// slab stays in L2 across kx and Px - kx and the components) rather than staged: without its
-// 33 KB the CTA's shared memory is the 64 KB of its nz lines, three CTAs per SM instead of two.
-template <int M, int MZ>
-__global__ void __launch_bounds__(256) k_wslab_yz(float2* __restrict__ ws,
-                                                  const float2* __restrict__ gs,
-                                                  const float2* __restrict__ twy,
-                                                  const float2* __restrict__ twz, SlabArgs a) {
-  extern __shared__ unsigned char smem_raw[];
-  float2* S = reinterpret_cast<float2*>(smem_raw);  // [z][32 M]
-  constexpr int P = 32 * M;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int kx = blockIdx.x, c = blockIdx.y;
-  const int fx = min(kx, a.Px - kx);
-  const float2* G = gs + (int64_t)fx * a.gz * a.gy;  // this kx's Ghat slab [fz][fy]
-  float2* X = ws + c * a.P3 + (int64_t)kx * a.nz * a.ny;  // [z][y]
-  for (int z = warp; z < a.nz; z += 8) {
-    float2 v[M];
-#pragma unroll
-    for (int n1 = 0; n1 < M; ++n1) {
-      const int y = lane + 32 * n1;
-      v[n1] = y < a.ny ? X[(int64_t)z * a.ny + y] : make_float2(0.f, 0.f);
-    }
-    wline_fwd<M>(v, twy, lane);
-#pragma unroll
-    for (int k1 = 0; k1 < M; ++k1) S[z * P + k1 * 32 + lane] = v[k1];
-  }
-  __syncthreads();
-  for (int pos = threadIdx.x; pos < P; pos += blockDim.x) {
-    const int ky = (pos >> 5) + M * brev_l<32>(pos & 31);
-    const int fy = min(ky, P - ky);
-    float2 v[MZ];
-#pragma unroll
-    for (int z = 0; z < MZ; ++z) v[z] = z < a.nz ? S[z * P + pos] : make_float2(0.f, 0.f);
-    dft_reg<float2, MZ>(v, twz, 1, false);
-#pragma unroll
-    for (int kz = 0; kz < MZ; ++kz) v[kz] = cmul(v[kz], __ldg(&G[min(kz, MZ - kz) * a.gy + fy]));
-    dft_reg<float2, MZ>(v, twz, 1, true);
-#pragma unroll
-    for (int z = 0; z < MZ; ++z)
-      if (z < a.nz) S[z * P + pos] = v[z];
-  }
-  __syncthreads();
-  for (int z = warp; z < a.nz; z += 8) {
-    float2 v[M];
-#pragma unroll
-    for (int k1 = 0; k1 < M; ++k1) v[k1] = S[z * P + k1 * 32 + lane];
-    wline_inv<M>(v, twy, lane);
-#pragma unroll
-    for (int n1 = 0; n1 < M; ++n1) {
-      const int y = lane + 32 * n1;
-      if (y < a.ny) X[(int64_t)z * a.ny + y] = v[n1];
-    }
-  }
-}
-
-// x inverse: the CTA reads X[c][kx][z][y0 .. y0 + 7] as 64-byte runs into the shared tile; warp
-// w takes row y0 + w from it in the transform's order, inverts it and writes the nx kept values
-template <int M>
-__global__ void __launch_bounds__(256) k_wslab_xinv(const float2* __restrict__ ws,
-                                                    float2* __restrict__ phi,
-                                                    const float2* __restrict__ twx, SlabArgs a) {
-  extern __shared__ float2 tile[];  // [8 rows][TS]
-  constexpr int P = 32 * M, TS = P + P / 32 + 1;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int y0 = blockIdx.x * 8, y = y0 + warp, z = blockIdx.y, c = blockIdx.z;
-  const int nr = min(8, a.ny - y0);
-  const float2* src = ws + c * a.P3 + (int64_t)z * a.ny + y0;
-  for (int i = threadIdx.x; i < 8 * P; i += blockDim.x) {
-    const int kx = i >> 3, r = i & 7;
-    if (r < nr) tile[r * TS + kx + (kx >> 5)] = src[(int64_t)kx * a.nz * a.ny + r];
-  }
-  __syncthreads();
-  if (y >= a.ny) return;  // warp-uniform
-  const int k2 = brev_l<32>(lane);
-  float2 v[M];
-#pragma unroll
-  for (int k1 = 0; k1 < M; ++k1) {
-    const int kx = k1 + M * k2;
-    v[k1] = tile[warp * TS + kx + (kx >> 5)];
-  }
-  wline_inv<M>(v, twx, lane);
-  float2* dst = phi + c * a.ng + ((int64_t)z * a.ny + y) * a.nx;
-#pragma unroll
-  for (int n1 = 0; n1 < M; ++n1) {
-    const int x = lane + 32 * n1;
-    if (x < a.nx) dst[x] = v[n1];
-  }
-}
-
 // Ghat octant [fz][fy][fx] -> [fx][fz][fy] for the y-z pass (one contiguous slab per kx)
 __global__ void k_ghat_slab(const float2* __restrict__ oct, int gx, int gy, int gz, float2* gs) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -1260,6 +1004,11 @@ bool slab_path(const aim_ctx* c) {
          slab_x_smem(Px) <= kSmemBudget && slab_yz_smem(Py, nz, Pz) <= kSmemBudget;
 }
 
+// and the two-pass form of fft_two.cu where it has the lengths
+static bool big_two_path(const aim_ctx* c) {
+  return plane_smem<float2>(c->gp[0], c->gp[1]) > kSmemBudget && two_path(c);
+}
+
 static int slab_conv(aim_ctx* c, PrecBuf<float>& b, const float2* sigma, float2* phi, int ncomp,
                      float2* ws, cudaStream_t s) {
   SlabArgs a;
@@ -1273,24 +1022,6 @@ static int slab_conv(aim_ctx* c, PrecBuf<float>& b, const float2* sigma, float2*
   a.gy = a.Py / 2 + 1; a.gz = a.Pz / 2 + 1;
   a.mag_Px = div_magic(a.Px); a.mag_Py = div_magic(a.Py); a.mag_ny = div_magic(a.ny);
   a.mag_RY = div_magic(kSlabRY);
-  // the warp-line forms: both in-plane lengths 1024 (or 512) and a z length the register DFT
-  // takes
-  if (a.Px == a.Py && (a.Px == 1024 || a.Px == 512) && a.nz <= 8 && a.Pz == 15) {
-    const dim3 gw((a.ny + 7) / 8, a.nz, ncomp);
-    const size_t ssm = (size_t)a.nz * a.Py * sizeof(float2);
-    const size_t tsm = 8 * (size_t)(a.Px + a.Px / 32 + 1) * sizeof(float2);  // the x passes' tile
-    if (a.Px == 1024) {
-      k_wslab_xfwd<32><<<gw, 256, tsm, s>>>(sigma, ws, b.tw[0], a);
-      k_wslab_yz<32, 15><<<dim3(a.Px, ncomp), 256, ssm, s>>>(ws, b.Gs, b.tw[1], b.tw[2], a);
-      k_wslab_xinv<32><<<gw, 256, tsm, s>>>(ws, phi, b.tw[0], a);
-    } else {
-      k_wslab_xfwd<16><<<gw, 256, tsm, s>>>(sigma, ws, b.tw[0], a);
-      k_wslab_yz<16, 15><<<dim3(a.Px, ncomp), 256, ssm, s>>>(ws, b.Gs, b.tw[1], b.tw[2], a);
-      k_wslab_xinv<16><<<gw, 256, tsm, s>>>(ws, phi, b.tw[0], a);
-    }
-    BEM_CUDA(cudaGetLastError());
-    return BEM_OK;
-  }
   const dim3 gx((a.ny + kSlabRY - 1) / kSlabRY, a.nz, ncomp);
   k_slab_xfwd<<<gx, 256, slab_x_smem(a.Px), s>>>(sigma, ws, b.tw[0], a);
   slab_yz_kernel(a.Pz)<<<dim3(a.Px, ncomp), 256, slab_yz_smem(a.Py, a.nz, a.Pz), s>>>(
@@ -1313,12 +1044,6 @@ int fft_init_attrs() {
   BEM_CUDA(cudaFuncSetAttribute(k_slab_xfwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   for (int pz : {8, 9, 10, 12, 15, 16, 0})
     BEM_CUDA(cudaFuncSetAttribute(slab_yz_kernel(pz), cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-  BEM_CUDA(cudaFuncSetAttribute(k_wslab_yz<32, 15>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-  BEM_CUDA(cudaFuncSetAttribute(k_wslab_xfwd<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-  BEM_CUDA(cudaFuncSetAttribute(k_wslab_xinv<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-  BEM_CUDA(cudaFuncSetAttribute(k_wslab_xfwd<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-  BEM_CUDA(cudaFuncSetAttribute(k_wslab_xinv<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-  BEM_CUDA(cudaFuncSetAttribute(k_wslab_yz<16, 15>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   BEM_CUDA(cudaFuncSetAttribute(k_slab_xinv, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   return BEM_OK;
 }
@@ -1394,6 +1119,7 @@ int fft_conv(aim_ctx* c, PrecBuf<R>& b, const typename C2<R>::T* sigma, typename
     return BEM_OK;
   }
   if constexpr (sizeof(V) == sizeof(float2)) {
+    if (two_path(c)) return two_conv(c, sigma, phi, ncomp, ws, s);
     if (b.Gs) return slab_conv(c, b, sigma, phi, ncomp, ws, s);
   }
   LinePass p{};
@@ -1508,7 +1234,10 @@ int make_ghat(aim_ctx* c) {
   if (rc == BEM_OK) rc = dalloc_t(c, &c->f32.Ghat, no);
   int zl = 0, zm = 0;
   if (rc == BEM_OK && reg_shape(Pz, &zl, &zm)) rc = dalloc_t(c, &c->f32.Gz, P3);
-  if (rc == BEM_OK && slab_path(c)) rc = dalloc_t(c, &c->f32.Gs, no);
+  if (rc == BEM_OK && (slab_path(c) || big_two_path(c))) {
+    rc = dalloc_t(c, &c->f32.Gs, no);
+    if (rc == BEM_OK && big_two_path(c)) rc = two_twiddles(c);
+  }
   if (rc == BEM_OK) {
     k_ghat_oct<<<(unsigned)((no + 255) / 256), 256>>>(G, Px, Py, Pz, 1.0 / (double)P3, c->f64.Ghat,
                                                       c->f32.Ghat);

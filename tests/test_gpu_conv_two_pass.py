@@ -1,0 +1,48 @@
+"""The grid step on grids beyond the plane passes, FP32, over the lengths the two-pass transforms take:
+every radix of the x and y passes, z in registers (Pz a radix) and as two passes (nz > 16), rows that
+are no multiple of eight, equal and unlike x and y, one to five components where the entry allows
+four. Against NumPy's FFT in 64 bits; 2e-6, the tolerance of the other FP32 convolution tests."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle import operators as op  # noqa: E402
+from paper_2108_03991_gb300 import api, synth  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2108_03991_gb300 import build
+    build.build()
+
+
+@pytest.mark.parametrize("n", [(128, 125, 8), (150, 90, 21), (113, 101, 9), (135, 144, 7), (203, 48, 33),
+                               (321, 37, 12), (76, 200, 40), (512, 61, 6), (97, 97, 16), (240, 162, 25),
+                               (313, 365, 8), (405, 75, 10)])
+def test_conv(n):
+    grid = synth.Grid(np.array([-1.1, -1.1, -1.1]), np.array([0.5, 0.4, 0.5]), np.array(n))
+    freq = 3e13  # kR up to a hundred: the phase of the grid kernel matters
+    ctx = api.Context(synth.bar_mesh(1.0, 1.0, 1.0, 0.5), grid, freq)
+    k0 = op.k0_of(freq)
+    P = [2 * v for v in n]
+    ax = [np.minimum(np.arange(p), p - np.arange(p)) * h for p, h in zip(P, grid.h)]
+    R = np.sqrt(ax[2][:, None, None] ** 2 + ax[1][None, :, None] ** 2 + ax[0][None, None, :] ** 2)
+    R[0, 0, 0] = 1.0
+    G = np.exp(-1j * k0 * R) / (4 * np.pi * R)
+    G[0, 0, 0] = 0
+    G = np.fft.fftn(G)
+    for ncomp in (1, 4) if n[2] < 20 else (3,):
+        s = synth.rand_cvec(ncomp * ctx.ng, 9).reshape(ncomp, n[2], n[1], n[0])
+        f = np.fft.ifftn(np.fft.fftn(s, s=(P[2], P[1], P[0]), axes=(1, 2, 3)) * G, axes=(1, 2, 3))
+        ref = f[:, :n[2], :n[1], :n[0]]
+        d = torch.from_numpy(s.astype(np.complex64).ravel()).cuda()
+        out = ctx.conv(d, ncomp=ncomp).cpu().numpy().reshape(s.shape)
+        inplace = ctx.conv(d, d, ncomp=ncomp).cpu().numpy().reshape(s.shape)
+        for c in range(ncomp):
+            assert np.linalg.norm(out[c] - ref[c]) <= 2e-6 * np.linalg.norm(ref[c])
+        assert np.array_equal(out, inplace)
+    ctx.close()
