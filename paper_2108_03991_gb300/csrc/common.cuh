@@ -62,6 +62,35 @@ __device__ __forceinline__ void cfma(float2& a, float2 b, float2 c) {
   a.y = fmaf(b.x, c.y, fmaf(b.y, c.x, a.y));
 }
 
+// a + b, a - b, c a + b (c real): in FP32 both parts in one packed instruction (add, fma .f32x2, each part
+// rounded as the scalar instruction does), which halves the issue slots of the additions
+__device__ __forceinline__ unsigned long long f2_pack(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+  return r;
+}
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(f2_pack(a)), "l"(f2_pack(b)));
+  return f2_unpack(r);
+}
+__device__ __forceinline__ float2 vfma(float c, float2 a, float2 b) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(f2_pack(make_float2(c, c))), "l"(f2_pack(a)), "l"(f2_pack(b)));
+  return f2_unpack(r);
+}
+__device__ __forceinline__ float2 vsub(float2 a, float2 b) { return vfma(-1.f, b, a); }
+__device__ __forceinline__ double2 vfma(double c, double2 a, double2 b) {
+  return make_double2(fma(c, a.x, b.x), fma(c, a.y, b.y));
+}
+__device__ __forceinline__ double2 vadd(double2 a, double2 b) { return cadd(a, b); }
+__device__ __forceinline__ double2 vsub(double2 a, double2 b) { return csub(a, b); }
+
 template <typename V> __device__ __forceinline__ V warp_sum(V v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -254,6 +283,7 @@ struct aim_ctx {
   bem::GemvPlan gplan64;  // FP64 products
   bem::GemvPlan gbg32, gbg64;  // e = Z h beside the AIM chain in the system matvec (few CTAs)
   bem::GemvPlan gpair;         // j = h - C h and e = Z h as one task list (both precisions)
+  bem::GemvPlan gm16;          // tasks of 16 rows (more than four right-hand sides: k_gemv_m8)
   bem::GemvPlan gmr;           // several right-hand sides: task list of 16-row tasks (k_gemv_mr)
   bem::GemvPlan gplan_auto;    // the autotuner's FP32 choice
   bem::GemvPlan gplan_alt[2];  // best plain and best staged FP32 plans (ncta = 0: none)

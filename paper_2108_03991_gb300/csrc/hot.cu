@@ -54,7 +54,7 @@ __device__ __forceinline__ void dot_range(const typename Vec16<R>::T* __restrict
           if constexpr (PAIR) {
             auto t = cmul(a0, mk(q.x, q.y));
             cfma(t, a1, mk(q.z, q.w));
-            acc[r] = cadd(acc[r], t);
+            acc[r] = vadd(acc[r], t);
           } else {
             cfma(acc[r], a0, mk(q.x, q.y));
             cfma(acc[r], a1, mk(q.z, q.w));
@@ -62,7 +62,7 @@ __device__ __forceinline__ void dot_range(const typename Vec16<R>::T* __restrict
         } else if (PAIR) {
           auto t = cmul(a0, __ldg(xb + r * vstride + col));
           if (col + 1 < n) cfma(t, a1, __ldg(xb + r * vstride + col + 1));
-          acc[r] = cadd(acc[r], t);
+          acc[r] = vadd(acc[r], t);
         } else {
           cfma(acc[r], a0, __ldg(xb + r * vstride + col));
           if (col + 1 < n) cfma(acc[r], a1, __ldg(xb + r * vstride + col + 1));
@@ -188,7 +188,7 @@ __device__ __forceinline__ void gemv_mr_task(const GemvTask& t, const typename C
           for (int k = 0; k < RB; ++k) {
             V p = cmul(mk(a[u][k].x, a[u][k].y), x0);
             if (two) cfma(p, mk(a[u][k].z, a[u][k].w), x1);
-            acc[k][r] = cadd(acc[k][r], p);
+            acc[k][r] = vadd(acc[k][r], p);
           }
         }
         continue;
@@ -274,6 +274,79 @@ template int run_gemv_mr<float>(const GemvPlan&, const float2*, const float2*, f
                                 const float2*, cudaStream_t);
 template int run_gemv_mr<double>(const GemvPlan&, const double2*, const double2*, double2*, int,
                                  int64_t, const double2*, cudaStream_t);
+
+// Five right-hand sides and more (FP32): a warp takes 4 rows and 8 right-hand sides, lanes along the
+// columns, so a 16-byte load of the matrix meets 8 vectors and every load of x serves 4 rows; the next
+// vector of each row is in flight while the current one is used. The two groups of 4 warps of a CTA
+// take the same 16 rows and neighbouring eights of right-hand sides (the second group's matrix loads
+// hit L1). Bound by the FP32 pipe (8 flops per entry and right-hand side). The 32 complex partial sums of a
+// warp meet in a reduce-scatter (62 shuffles instead of 320), which leaves row k and right-hand side r
+// of the tile in lane 8 k + r. y_r = A x_r for r < nrhs.
+constexpr int kM8 = 8;
+__device__ __forceinline__ void gemv_m8_task(const GemvTask& t, const float2* __restrict__ A,
+                                             const float2* __restrict__ x, float2* __restrict__ y,
+                                             int64_t vstride, int nrhs, int rg) {
+  const int warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+  const int r0 = t.row0 + 4 * warp, nr = min(4, t.row0 + t.nrows - r0), R = min(kM8, nrhs - kM8 * rg);
+  if (nr <= 0 || R <= 0) return;
+  x += (int64_t)kM8 * rg * vstride + t.xoff;
+  y += (int64_t)kM8 * rg * vstride + t.xoff;
+  const float4* arow[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    arow[k] = reinterpret_cast<const float4*>(A + t.aoff + (int64_t)(r0 + min(k, nr - 1)) * t.ld);
+  const float2* xr[kM8];  // a missing right-hand side repeats the last one
+#pragma unroll
+  for (int r = 0; r < kM8; ++r) xr[r] = x + min(r, R - 1) * vstride;
+  float2 acc[4 * kM8];
+#pragma unroll
+  for (int i = 0; i < 4 * kM8; ++i) acc[i] = make_float2(0.f, 0.f);
+  const int nv = (t.n + 1) / 2;
+  float4 a[4];
+  if (lane < nv) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = __ldg(arow[k] + lane);
+  }
+  for (int v = lane; v < nv; v += 32) {
+    float4 b[4];
+    const bool more = v + 32 < nv;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) b[k] = more ? __ldg(arow[k] + v + 32) : make_float4(0.f, 0.f, 0.f, 0.f);
+    const bool two = 2 * v + 1 < t.n;
+#pragma unroll
+    for (int r = 0; r < kM8; ++r) {
+      const float2 x0 = __ldg(xr[r] + 2 * v), x1 = two ? __ldg(xr[r] + 2 * v + 1) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        float2 p = cmul(make_float2(a[k].x, a[k].y), x0);  // the two entries first, as in dot_range
+        if (two) cfma(p, make_float2(a[k].z, a[k].w), x1);
+        acc[kM8 * k + r] = vadd(acc[kM8 * k + r], p);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) a[k] = b[k];
+  }
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) {
+    const bool up = lane & m;
+#pragma unroll
+    for (int i = 0; i < m; ++i) {
+      const float2 keep = up ? acc[m + i] : acc[i], send = up ? acc[i] : acc[m + i];
+      acc[i] = vadd(keep, make_float2(__shfl_xor_sync(0xffffffffu, send.x, m), __shfl_xor_sync(0xffffffffu, send.y, m)));
+    }
+  }
+  const int k = lane / kM8, r = lane % kM8;
+  if (k < nr && r < R) y[(int64_t)r * vstride + r0 + k] = acc[0];
+}
+
+// grid: tasks of 16 rows, pairs of eights of right-hand sides, the matrices (A0 to y0, A1 to y1)
+__global__ void __launch_bounds__(256, 2) k_gemv_m8(const GemvTask* __restrict__ tasks, const float2* __restrict__ A0,
+                                                    const float2* __restrict__ A1, const float2* __restrict__ x,
+                                                    float2* __restrict__ y0, float2* __restrict__ y1,
+                                                    int64_t vstride, int nrhs) {
+  gemv_m8_task(tasks[blockIdx.x], blockIdx.z ? A1 : A0, x, blockIdx.z ? y1 : y0, vstride, nrhs,
+               2 * blockIdx.y + (threadIdx.x >> 7));
+}
 
 // Paired task list: two block-diagonal matrices of the same layout applied to one x in one
 // launch; a task with sel = 0 computes y0 = hsub - A0 x (or A0 x) on its rows, sel = 1
@@ -732,12 +805,22 @@ __global__ void __launch_bounds__(128)
   gemv_mr_task<R, NR, 4, true>(blk_task(tab, 16), A, x, y, vstride, nullptr);
 }
 
+template <int CAP>
+__global__ void __launch_bounds__(256, 2)
+    k_gemv_blk_m8(const __grid_constant__ BlkTab<CAP> tab, const float2* __restrict__ A,
+                  const float2* __restrict__ x, float2* __restrict__ y, int64_t vstride, int nrhs) {
+  gemv_m8_task(blk_task(tab, 16), A, x, y, vstride, nrhs, 2 * blockIdx.y + (threadIdx.x >> 7));
+}
+
 template <typename R, int CAP>
 static int launch_blk(const BlkTab<CAP>& tab, unsigned ntask, const typename C2<R>::T* A,
                       const typename C2<R>::T* x, typename C2<R>::T* y, int nrhs, int64_t vs,
                       cudaStream_t s) {
   if (nrhs == 1) {
     k_gemv_blk<R, CAP><<<ntask, 128, 0, s>>>(tab, A, x, y);
+  } else if (sizeof(R) == 4 && nrhs > 4) {
+    if constexpr (sizeof(R) == 4)
+      k_gemv_blk_m8<CAP><<<dim3(ntask, (nrhs + 15) / 16), nrhs > kM8 ? 256 : 128, 0, s>>>(tab, A, x, y, vs, nrhs);
   } else {
     for (int r0 = 0; r0 < nrhs; r0 += 4) {
       const int64_t o = r0 * vs;
@@ -1563,6 +1646,22 @@ int internal(aim_ctx* c, const void* hv, void* ev, void* heqv, int nrhs, cudaStr
   typedef typename C2<R>::T V;
   PrecBuf<R>& b = buf<R>(c);
   const GemvPlan& gp = sizeof(R) == 4 ? c->gplan : c->gplan64;
+  if constexpr (sizeof(R) == 4) {
+    // more than four right-hand sides: eight at a time (k_gemv_m8). Six bars of 240-1,920 edges, Z and
+    // C (us): 337 -> 117 at 16, 2,719 -> 858 at 128; one bar of 2,016 163 -> 42, 1,315 -> 268
+    if (nrhs > 4 && c->gm16.ntasks > 0 && !(ev && c->zsp_on)) {
+      const V* h = (const V*)hv;
+      for (int g = 0; g < nrhs; g += 16 * 65535) {  // gridDim.y
+        const int n = std::min(16 * 65535, nrhs - g);
+        const int64_t o = (int64_t)g * c->ne;
+        V *e = ev ? (V*)ev + o : nullptr, *q = heqv ? (V*)heqv + o : nullptr;
+        k_gemv_m8<<<dim3(c->gm16.ntasks, (n + 15) / 16, ev && heqv ? 2 : 1), n > kM8 ? 256 : 128, 0, s>>>(
+            c->gm16.tasks, ev ? b.Z : b.C, b.C, h + o, ev ? e : q, q, c->ne, n);
+      }
+      BEM_CUDA(cudaGetLastError());
+      return BEM_OK;
+    }
+  }
   if (!ev) {
   } else if (c->zsp_on) {  // e = Z_s h, the sparse internal operator
     BEM_TRY(zsp_apply<R>(c, (const V*)hv, (V*)ev, nrhs, c->ne, c->ne, s));

@@ -1011,6 +1011,7 @@ int tune_matvec_schedule(aim_ctx* c) {
     cudaFree(yy);
     BEM_CUDA(cudaGetLastError());
     c->gmr = tm[1] < tm[0] ? cand[1] : cand[0];
+    c->gm16 = cand[0];
   }
   // the last two entries stand for the serial schedules (e = Z h after j's GEMV with its
   // launch shape; both in one paired launch)

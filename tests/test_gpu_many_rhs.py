@@ -1,0 +1,52 @@
+"""More than four right-hand sides through the FP32 block products (eight at a time, pairs of eights
+per CTA, 4 rows per warp): counts around 4, 8 and 16, blocks whose size is odd, below a task of 16
+rows and no multiple of it, both outputs or one. internal_apply against the FP64 product of the same
+context, bem_blockdiag_gemv against NumPy; C32 1e-5 as the other GEMV tests."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_2108_03991_gb300 import api, synth  # noqa: E402
+
+COUNTS = [5, 8, 9, 16, 17, 31, 33]
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2108_03991_gb300 import build
+    build.build()
+    mesh = synth.small_bars(3, 3.0)
+    c = api.Context(mesh, synth.grid_box(mesh, 0.5), 10e9)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("nrhs", COUNTS)
+def test_internal(ctx, nrhs):
+    h = torch.from_numpy(synth.rand_cvec(nrhs * ctx.ne, 80 + nrhs).astype(np.complex64)).cuda()
+    e, q = ctx.internal(h, nrhs=nrhs)
+    e1, _ = ctx.internal(h, nrhs=nrhs, want_heq=False)
+    _, q1 = ctx.internal(h, nrhs=nrhs, want_e=False)
+    er, qr = ctx.internal(h.to(torch.complex128), nrhs=nrhs, prec=api.BEM_C64)
+    assert torch.equal(e, e1) and torch.equal(q, q1)
+    for out, ref in ((e, er), (q, qr)):
+        d = (out - ref).view(nrhs, -1).norm(dim=1)
+        assert bool((d <= 1e-5 * ref.view(nrhs, -1).norm(dim=1)).all())
+
+
+@pytest.mark.parametrize("nrhs", COUNTS)
+def test_blocks(ctx, nrhs):
+    sizes = [1, 2, 15, 16, 17, 63, 65, 130, 257]
+    blocks = synth.rand_blocks(sizes, 7)
+    N = sum(sizes)
+    x = synth.rand_cvec(nrhs * N, 90 + nrhs).reshape(nrhs, N)
+    ref = np.concatenate([x[:, o:o + B.shape[0]] @ B.T
+                          for o, B in zip(np.cumsum([0] + sizes), blocks)], axis=1)
+    A = torch.from_numpy(api.pack_blocks(blocks, np.complex64)).cuda()
+    xd = torch.from_numpy(x.astype(np.complex64).ravel()).cuda()
+    y = api.blockdiag_gemv(sizes, A, xd, torch.empty_like(xd), nrhs).cpu().numpy().reshape(nrhs, N)
+    assert np.all(np.linalg.norm(y - ref, axis=1) <= 1e-5 * np.linalg.norm(ref, axis=1))
