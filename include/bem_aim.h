@@ -130,7 +130,9 @@ int aim_info(const aim_ctx* ctx, int64_t* info, int n);
  * at most 256, and Z_s h must match the dense Z h to 1e-8 at set-up (FP64, one probe vector).
  * Then e = Z_s h = -(1/(j k0 eps_rc)) L_s^{-1}(K_s + I_x/2) h replaces e = Z h in aim_matvec,
  * internal_apply and bem_solve (C = Y_eq Z stays dense), and is on after aim_setup. on = 0
- * selects the dense Z again, on = 1 the sparse form (BEM_EINVAL when none was built).
+ * selects the dense Z again, on = 1 the sparse form (BEM_EINVAL when none was built). The FP64
+ * system products (aim_matvec, aim_matvec_batch, bem_solve's residuals) of few objects take the
+ * dense Z also then: where it was the faster one at set-up and the two agreed to 1e-13.
  * Synchronises the device; captured matvec graphs are rebuilt on next use. */
 int aim_internal_sparse(aim_ctx* ctx, int on);
 

@@ -1371,7 +1371,7 @@ int matvec_batch(aim_ctx* c, const void* xv, void* yv, int nrhs, cudaStream_t s)
   near_e_kernel<R>(c)<<<dim3(nb(ne, 8), nrhs), 256, 0, c->side>>>(c->d_rowA, c->d_lstA, c->d_clA, b.LA, b.bj, ne, b.ban,
                                                            N, ne);
   BEM_CUDA(cudaEventRecord(c->ev_join, c->side));
-  if (c->zsp_on)  // e_r = Z_s h_r, the sparse internal operator
+  if (zsp_used<R>(c, nrhs))  // e_r = Z_s h_r, the sparse internal operator
     BEM_TRY(zsp_apply<R>(c, x, b.be, nrhs, N, N, s));
   else
     BEM_TRY(gemv(b.Z, b.be, nullptr));  // e_r = Z h_r
@@ -1466,7 +1466,8 @@ int matvec(aim_ctx* c, int which, const void* xv, void* yv, cudaStream_t s) {
     const V* h = x;
     const V* q = x + ne;
     V* sq = b.sigma + 3 * ng;
-    const int za = c->zsp_on ? 0 : c->z_after;
+    const bool zsp = zsp_used<R>(c, 1);
+    const int za = zsp ? 0 : c->z_after;
     BEM_CUDA(cudaEventRecord(c->ev_fork, s));
     BEM_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
     if (za < 2) BEM_CUDA(cudaStreamWaitEvent(c->zside, c->ev_fork, 0));
@@ -1476,7 +1477,7 @@ int matvec(aim_ctx* c, int which, const void* xv, void* yv, cudaStream_t s) {
                                                 nt, nx, ny, b.p, 0, 0, 0);
     const GemvPlan& gp = sizeof(R) == 4 ? c->gplan : c->gplan64;
     const GemvPlan& gb = sizeof(R) == 4 ? c->gbg32 : c->gbg64;
-    if (c->zsp_on) BEM_TRY(zsp_apply<R>(c, h, b.e, 1, ne, ne, c->zside));
+    if (zsp) BEM_TRY(zsp_apply<R>(c, h, b.e, 1, ne, ne, c->zside));
     if (za == 3)  // j = h - C h and e = Z h in one launch
       BEM_TRY(run_gemv_pair<R>(c->gpair, b.C, b.Z, h, b.j, b.e, h, s));
     else
@@ -1488,7 +1489,7 @@ int matvec(aim_ctx* c, int which, const void* xv, void* yv, cudaStream_t s) {
     BEM_CUDA(cudaEventRecord(c->ev_join, c->side));
     if (za == 2) {  // e = Z h right after j's GEMV on the main stream, whole GPU
       BEM_TRY(run_gemv_plan<R>(gp, b.Z, h, b.e, 1, ne, nullptr, s));
-    } else if (za != 3 && !c->zsp_on) {
+    } else if (za != 3 && !zsp) {
       if (za)  // e = Z h once j is out, beside the AIM chain only
         BEM_CUDA(cudaStreamWaitEvent(c->zside, c->ev_c, 0));
       BEM_TRY(run_gemv_plan<R>(gb, b.Z, h, b.e, 1, ne, nullptr, c->zside));

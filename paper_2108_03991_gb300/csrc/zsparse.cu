@@ -40,6 +40,7 @@ constexpr int kZspW32 = 32, kZspW64 = 16, kZspW64s = 8;
 constexpr int kZspRing = 256;        // second accumulator, a ring over rows (>= 192 + 32)
 constexpr int kZspStages = 3;        // slabs in flight (2 where shared memory leaves no room)
 constexpr double kZspCheck = 1e-8;   // set-up check of Z_s h against Z h
+constexpr double kZspSame = 1e-13;  // below it Z_s h and Z h are the same product to FP64 rounding
 constexpr double kTwoPi = 6.283185307179586476925;
 
 struct ZspObj {
@@ -765,6 +766,27 @@ int zsp_check(aim_ctx* c) {
     return BEM_OK;
   }
   c->zsp_on = true;
+  // FP64: a ring's substitutions are bound by the FP64 rate of the one SM they run on, the dense
+  // product by the whole GPU's, so few objects are faster dense (4 rings of 912 edges 35 us against
+  // 413, 36 rings 282 / 453, 256 rings 2,000 / 979). The system matvec takes the faster one where both
+  // are the same product to rounding.
+  if (worst <= kZspSame) {
+    cudaEvent_t ev[3];
+    for (cudaEvent_t& q : ev) BEM_CUDA(cudaEventCreate(&q));
+    cudaEventRecord(ev[0], 0);
+    rc = zsp_apply<double>(c, h, e1, 1, ne, ne, 0);
+    cudaEventRecord(ev[1], 0);
+    if (rc == BEM_OK) rc = run_gemv_plan<double>(c->gplan64, c->f64.Z, h, e2, 1, ne, nullptr, 0);
+    cudaEventRecord(ev[2], 0);
+    cudaError_t sync = cudaEventSynchronize(ev[2]);
+    if (rc == BEM_OK && sync == cudaSuccess) {
+      cudaEventElapsedTime(&c->zsp64_ms[0], ev[0], ev[1]);
+      cudaEventElapsedTime(&c->zsp64_ms[1], ev[1], ev[2]);
+    }
+    for (cudaEvent_t& q : ev) cudaEventDestroy(q);
+    BEM_TRY(rc);
+    BEM_CUDA(sync);
+  }
   return BEM_OK;
 }
 
