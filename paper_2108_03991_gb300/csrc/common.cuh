@@ -453,6 +453,10 @@ int make_ghat(aim_ctx* c);
 // the convolution
 bool two_path(const aim_ctx* c);
 int two_twiddles(aim_ctx* c);
+int two_init_attrs();
+bool two_z_radix(int Pz);  // whether two_z has it
+// the z pass of the plane passes for a Pz that is a radix (true when it ran)
+bool two_z(aim_ctx* c, float2* ws, int ncomp, cudaStream_t s);
 int two_conv(aim_ctx* c, const float2* sigma, float2* phi, int ncomp, float2* ws, cudaStream_t s);
 int rhs_plane_wave(aim_ctx* c, const double* pol, const double* kh, void* b, int prec,
                    cudaStream_t st);

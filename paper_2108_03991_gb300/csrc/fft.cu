@@ -789,6 +789,7 @@ __global__ void __launch_bounds__(256) k_lines(const V* in, V* out, const V* __r
 }
 
 static constexpr size_t kSmemBudget = 200 * 1024;
+static constexpr int kFftSms = 152;
 
 template <typename V>
 static int launch_lines(const V* in, V* out, const V* tw, const V* ghat, LinePass p, int n2,
@@ -801,6 +802,8 @@ static int launch_lines(const V* in, V* out, const V* tw, const V* ghat, LinePas
   }
   int TL = (int)std::min<size_t>(16, (avail - p.P) / (2 * pitch));
   TL = std::max(1, std::min(TL, p.n0));
+  // fewer lines per CTA where the launch would leave SMs without one
+  while (TL > 4 && (int64_t)((p.n0 + TL - 1) / TL) * p.n1 * n2 < 2 * kFftSms) TL = (TL + 1) / 2;
   p.TL = TL;
   p.mag_P = div_magic(p.P);
   p.mag_TL = div_magic(TL);
@@ -1004,11 +1007,6 @@ bool slab_path(const aim_ctx* c) {
          slab_x_smem(Px) <= kSmemBudget && slab_yz_smem(Py, nz, Pz) <= kSmemBudget;
 }
 
-// and the two-pass form of fft_two.cu where it has the lengths
-static bool big_two_path(const aim_ctx* c) {
-  return plane_smem<float2>(c->gp[0], c->gp[1]) > kSmemBudget && two_path(c);
-}
-
 static int slab_conv(aim_ctx* c, PrecBuf<float>& b, const float2* sigma, float2* phi, int ncomp,
                      float2* ws, cudaStream_t s) {
   SlabArgs a;
@@ -1032,6 +1030,7 @@ static int slab_conv(aim_ctx* c, PrecBuf<float>& b, const float2* sigma, float2*
 }
 
 int fft_init_attrs() {
+  BEM_TRY(two_init_attrs());
   const int lim = (int)kSmemBudget;
   BEM_CUDA(cudaFuncSetAttribute(k_lines<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   BEM_CUDA(cudaFuncSetAttribute(k_lines<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
@@ -1065,6 +1064,18 @@ int make_twiddles(aim_ctx* c, PrecBuf<R>& b) {
 template int make_twiddles<float>(aim_ctx*, PrecBuf<float>&);
 template int make_twiddles<double>(aim_ctx*, PrecBuf<double>&);
 
+// FP32: the two-pass form of fft_two.cu where it has the lengths, but for small planes with a register
+// z pass: there the plane passes' two launches of one CTA per plane are the shorter chain (us, three
+// components, plane / two-pass: 25^3 10.3 / 11.5, 32^3 10.4 / 11.7, 40 x 40 x 18 8.2 / 11.1; 60 x 40 x 80
+// 17.4 / 14.8, 64 x 64 x 15 14.6 / 10.5, 96 x 96 x 15 26.6 / 11.9, 72 x 72 x 160 31.2 / 26.9, 100^3
+// 65 / 27; with the shared-memory z pass 15 x 15 x 90 12.7 / 10.1).
+static bool use_two(const aim_ctx* c) {
+  const int Px = c->gp[0], Py = c->gp[1], Pz = c->gp[2];
+  int l, m;
+  const bool small = plane_smem<float2>(Px, Py) <= kSmemBudget && Px * Py < 2000;
+  return two_path(c) && !(small && (reg_shape(Pz, &l, &m) || two_z_radix(Pz)));
+}
+
 template <typename R>
 int fft_conv(aim_ctx* c, PrecBuf<R>& b, const typename C2<R>::T* sigma, typename C2<R>::T* phi,
              int ncomp, typename C2<R>::T* ws, cudaStream_t s) {
@@ -1072,8 +1083,15 @@ int fft_conv(aim_ctx* c, PrecBuf<R>& b, const typename C2<R>::T* sigma, typename
   const int nx = c->gn[0], ny = c->gn[1], nz = c->gn[2];
   const int Px = c->gp[0], Py = c->gp[1], Pz = c->gp[2];
   const int64_t P3 = (int64_t)Px * Py * Pz, ng = c->ng;
+  if constexpr (sizeof(V) == sizeof(float2)) {
+    if (b.tt[0]) return two_conv(c, sigma, phi, ncomp, ws, s);
+  }
   const size_t psm = plane_smem<V>(Px, Py);
-  if (psm <= kSmemBudget) {
+  // FP64: a plane's transforms are bound by the FP64 rate of the one SM they run on (64 x 64: 37 us a
+  // pass), so few large planes go as lines over the whole GPU (three components of 64 x 64 x 15 99 -> 70
+  // us; 32 x 32 planes take longer that way, 38 -> 46)
+  const bool lines64 = sizeof(R) == 8 && nz * ncomp <= kFftSms / 2 && Px * Py >= 1600;
+  if (psm <= kSmemBudget && !lines64) {
     PlaneArgs a;
     a.nx = nx; a.ny = ny; a.nz = nz; a.Px = Px; a.Py = Py; a.Pz = Pz;
     a.ng = ng; a.P3 = P3;
@@ -1082,6 +1100,9 @@ int fft_conv(aim_ctx* c, PrecBuf<R>& b, const typename C2<R>::T* sigma, typename
     const size_t avail = 64 * 1024 / sizeof(V);
     const size_t zp = sw_len(Pz);
     a.TL = (int)std::max<size_t>(1, std::min<size_t>(16, (avail - Pz) / (2 * zp)));
+    // fewer lines per CTA where the launch would leave SMs without one (FP64 15 x 15 x 90: 34 us with 16
+    // lines on 45 CTAs)
+    while (a.TL > 2 && (int64_t)((Px + a.TL - 1) / a.TL) * Py * ncomp < kFftSms) a.TL = (a.TL + 1) / 2;
     a.mag_Px = div_magic(Px);
     a.mag_nx = div_magic(nx);
     a.mag_TL = div_magic(a.TL);
@@ -1107,6 +1128,11 @@ int fft_conv(aim_ctx* c, PrecBuf<R>& b, const typename C2<R>::T* sigma, typename
         launch_zreg<V>(zl, zm, dim3((Px + per - 1) / per, Py, ncomp), s, ws, b.Ghat, b.Gz, b.tw[2], a);
       }
     }
+    if constexpr (sizeof(V) == sizeof(float2)) {
+      if (!z_done) {  // a line per thread where Pz is a radix
+        z_done = two_z(c, ws, ncomp, s);
+      }
+    }
     if (!z_done)
       k_zfused<V><<<dim3((Px + a.TL - 1) / a.TL, Py, ncomp), 256, zsm, s>>>(ws, b.Ghat, b.tw[2], a);
     if constexpr (sizeof(V) == sizeof(float2)) {
@@ -1119,7 +1145,6 @@ int fft_conv(aim_ctx* c, PrecBuf<R>& b, const typename C2<R>::T* sigma, typename
     return BEM_OK;
   }
   if constexpr (sizeof(V) == sizeof(float2)) {
-    if (two_path(c)) return two_conv(c, sigma, phi, ncomp, ws, s);
     if (b.Gs) return slab_conv(c, b, sigma, phi, ncomp, ws, s);
   }
   LinePass p{};
@@ -1233,10 +1258,10 @@ int make_ghat(aim_ctx* c) {
   if (rc == BEM_OK) rc = dalloc_t(c, &c->f64.Ghat, no);
   if (rc == BEM_OK) rc = dalloc_t(c, &c->f32.Ghat, no);
   int zl = 0, zm = 0;
-  if (rc == BEM_OK && reg_shape(Pz, &zl, &zm)) rc = dalloc_t(c, &c->f32.Gz, P3);
-  if (rc == BEM_OK && (slab_path(c) || big_two_path(c))) {
+  if (rc == BEM_OK && !use_two(c) && reg_shape(Pz, &zl, &zm)) rc = dalloc_t(c, &c->f32.Gz, P3);
+  if (rc == BEM_OK && (slab_path(c) || use_two(c))) {
     rc = dalloc_t(c, &c->f32.Gs, no);
-    if (rc == BEM_OK && big_two_path(c)) rc = two_twiddles(c);
+    if (rc == BEM_OK && use_two(c)) rc = two_twiddles(c);
   }
   if (rc == BEM_OK) {
     k_ghat_oct<<<(unsigned)((no + 255) / 256), 256>>>(G, Px, Py, Pz, 1.0 / (double)P3, c->f64.Ghat,

@@ -1,5 +1,4 @@
-// The grid step's convolution in FP32 for grids whose padded x-y plane does not fit shared memory
-// (the split-ring array's 1024 x 1024 planes among them): every transform of length P = A B is two
+// The grid step's convolution in FP32 for all but small grids (use_two in fft.cu): every transform of length P = A B is two
 // register passes with one trip through shared memory between them,
 //   n = b + B a, k = ka + A kb:  X[k] = sum_b W_P^(b ka) W_B^(b kb) sum_a W_A^(a ka) x[n],
 // the A-point transforms over a with the twiddles W_P^(b ka), then the B-point transforms over b, both
@@ -14,8 +13,8 @@
 //   x inverse : the mirror of the first launch
 // Bound by the workspace's traffic (L2 or HBM) and the shared-memory trips: a value crosses shared
 // memory 2 times per line where the forms before (shuffle stages in a warp, 10 shuffles a value;
-// radix-8 Stockham passes with a trip per stage; five passes over the whole padded grid where nz > 16)
-// took 5 to 25.
+// radix-8 Stockham passes with a trip per stage; five passes over the whole padded grid where nz > 16;
+// or a whole plane per CTA, which leaves SMs without one) took 5 to 25.
 // Three components (us): 512 x 512 x 8 399 -> 326, 256 x 256 x 8 101 -> 92, 150 x 90 x 21 242 -> 65, 400 x 300 x
 // 12 1,722 -> 219, 96 x 80 x 72 284 -> 100, 200 x 30 x 9 169 -> 26.
 // Not kept: every pass through one loop over shared memory, each radix's code once per kernel (782 us
@@ -523,6 +522,53 @@ int two_twiddles(aim_ctx* c) {
   return BEM_OK;
 }
 
+int two_init_attrs() {
+  for (const void* f : {(const void*)k_two_xfwd<16>, (const void*)k_two_xfwd<32>, (const void*)k_two_yz<16>,
+                        (const void*)k_two_yz<32>, (const void*)k_two_xinv<16>, (const void*)k_two_xinv<32>})
+    BEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTwoSmem));
+  return BEM_OK;
+}
+
+// z pass over the padded planes [z][Py][Px] of the plane passes: a thread has one (x, y) line of M = Pz
+// points in registers (neighbouring threads neighbouring x: every load and store is coalesced, where
+// the shared-memory passes stage a tile and synchronise at every stage). The three passes of 64 x 64 x
+// 15, three components, 18.7 -> 14.6 us, of 40 x 40 x 18 10.9 -> 8.2.
+template <int M>
+__global__ void __launch_bounds__(64) k_two_z(float2* __restrict__ ws, const float2* __restrict__ ghat, int Px, int Py,
+                                              int nz, int64_t P3) {
+  const int i = blockIdx.x * 64 + threadIdx.x;
+  if (i >= Px * Py) return;
+  const int y = i / Px, x = i - y * Px, gx = Px / 2 + 1, gy = Py / 2 + 1;
+  const int64_t plane = (int64_t)Px * Py;
+  float2* s = ws + blockIdx.y * P3 + i;
+  const float2* g = ghat + (int64_t)min(y, Py - y) * gx + min(x, Px - x);
+  float2 v[M];
+#pragma unroll
+  for (int z = 0; z < held(M); ++z) v[z] = z < nz ? s[z * plane] : make_float2(0.f, 0.f);
+  dft<M, false, held(M)>(v);
+#pragma unroll
+  for (int z = 0; z < M; ++z) v[z] = cmul(v[z], __ldg(g + (int64_t)min(z, M - z) * gy * gx));
+  dft<M, true>(v);
+#pragma unroll
+  for (int z = 0; z < held(M); ++z)
+    if (z < nz) s[z * plane] = v[z];
+}
+
+bool two_z_radix(int Pz) { return is_radix(Pz); }
+
+bool two_z(aim_ctx* c, float2* ws, int ncomp, cudaStream_t s) {
+  const int Px = c->gp[0], Py = c->gp[1], Pz = c->gp[2];
+  const dim3 grid((Px * Py + 63) / 64, ncomp);
+  switch (Pz) {
+#define BEM_C(M)                                                                                                   \
+  case M: k_two_z<M><<<grid, 64, 0, s>>>(ws, c->f32.Ghat, Px, Py, c->gn[2], (int64_t)Px * Py * Pz); return true;
+    BEM_RADIX16(BEM_C)
+    BEM_RADIX32(BEM_C)
+#undef BEM_C
+    default: return false;
+  }
+}
+
 template <int CX, int CY>
 static int two_launch(aim_ctx* c, const TwoArgs& p, size_t xsm, size_t ysm, const float2* sigma, float2* phi,
                       int ncomp, float2* ws, cudaStream_t s) {
@@ -531,10 +577,6 @@ static int two_launch(aim_ctx* c, const TwoArgs& p, size_t xsm, size_t ysm, cons
   // threads of the y-z pass: 512 where shared memory leaves room for one CTA per SM
   const int ty = ysm > 100 * 1024 ? 512 : 256;
   const int tx = std::max(64, std::min(256, (int)round_up(kTwoRows * p.x.A, 32)));
-  // per call: the attribute belongs to the current device
-  BEM_CUDA(cudaFuncSetAttribute(k_two_xfwd<CX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTwoSmem));
-  BEM_CUDA(cudaFuncSetAttribute(k_two_xinv<CX>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTwoSmem));
-  BEM_CUDA(cudaFuncSetAttribute(k_two_yz<CY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTwoSmem));
   k_two_xfwd<CX><<<gx, tx, xsm, s>>>(sigma, ws, b.tt[0], p);
   k_two_yz<CY><<<dim3((p.x.P + p.nk - 1) / p.nk, ncomp), ty, ysm, s>>>(ws, b.Gs, b.tt[1], b.tt[2], p);
   k_two_xinv<CX><<<gx, tx, xsm, s>>>(ws, phi, b.tt[0], p);

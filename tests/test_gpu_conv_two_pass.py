@@ -46,3 +46,33 @@ def test_conv(n):
             assert np.linalg.norm(out[c] - ref[c]) <= 2e-6 * np.linalg.norm(ref[c])
         assert np.array_equal(out, inplace)
     ctx.close()
+
+
+def _reference(ctx, grid, freq, n, s):
+    k0 = op.k0_of(freq)
+    P = [2 * v for v in n]
+    ax = [np.minimum(np.arange(p), p - np.arange(p)) * h for p, h in zip(P, grid.h)]
+    R = np.sqrt(ax[2][:, None, None] ** 2 + ax[1][None, :, None] ** 2 + ax[0][None, None, :] ** 2)
+    R[0, 0, 0] = 1.0
+    G = np.exp(-1j * k0 * R) / (4 * np.pi * R)
+    G[0, 0, 0] = 0
+    f = np.fft.ifftn(np.fft.fftn(s, s=(P[2], P[1], P[0]), axes=(1, 2, 3)) * np.fft.fftn(G), axes=(1, 2, 3))
+    return f[:, :n[2], :n[1], :n[0]]
+
+
+@pytest.mark.parametrize("prec,n", [(api.BEM_C32, n) for n in ((7, 7, 43), (12, 11, 8), (20, 20, 9), (10, 9, 13),
+                                                                (8, 16, 16), (18, 18, 14), (23, 41, 8))] +
+                         [(api.BEM_C64, n) for n in ((7, 7, 43), (20, 20, 8), (24, 21, 9), (40, 33, 8))])
+def test_small_planes(prec, n):
+    """Small planes with a z line per thread (Pz a radix) or the shared-memory z pass, the first sizes of
+    the two-pass form, and FP64 planes as lines; C32 2e-6, C64 1e-12 as the other convolution tests."""
+    grid = synth.Grid(np.array([-1.1, -1.1, -1.1]), np.array([0.5, 0.4, 0.5]), np.array(n))
+    freq = 3e13
+    ctx = api.Context(synth.bar_mesh(1.0, 1.0, 1.0, 0.5), grid, freq)
+    s = synth.rand_cvec(3 * ctx.ng, 11).reshape(3, n[2], n[1], n[0])
+    ref = _reference(ctx, grid, freq, n, s)
+    out = ctx.conv(torch.from_numpy(s.ravel()).to(api.cdtype(prec)).cuda(), ncomp=3, prec=prec)
+    out = out.cpu().numpy().reshape(s.shape)
+    for c in range(3):
+        assert np.linalg.norm(out[c] - ref[c]) <= (2e-6 if prec == api.BEM_C32 else 1e-12) * np.linalg.norm(ref[c])
+    ctx.close()
