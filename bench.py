@@ -519,7 +519,7 @@ def bar_array_section(args, api, synth, torch, np, dev):
 
 def tensor_core_section(ctx, api, synth, torch, np, dev, hbm, reps=10):
     """h_eq = C h for R right-hand sides at once (C = Y_eq Z, complex FP32): the tensor-core
-    product (one pass over C per 128 right-hand sides, TF32 with the hi/lo split) against the
+    product (one pass over C per 128 right-hand sides, scaled FP16 hi and lo parts) against the
     block GEMV (one pass per 4), both through the library; the two agree to FP32 rounding. Per
     R: ms per product, C's bytes over that time, and the complex flops 8 sum n_i^2 R over it."""
     ZY = ctx.zy_bytes_c32 // 2
@@ -546,7 +546,7 @@ def tensor_core_section(ctx, api, synth, torch, np, dev, hbm, reps=10):
         t_tc = timed(lambda: ctx.internal_tc(h, None, y_tc, nrhs=R, want_e=False))
         t_mv = timed(lambda: ctx.internal(h, None, y_mv, nrhs=R, prec=api.BEM_C32, want_e=False))
         d = float(torch.linalg.vector_norm(y_tc - y_mv) / torch.linalg.vector_norm(y_mv))
-        ctx.tc_variant(1)  # the raw right-hand sides split in shared memory (half the packed bytes)
+        ctx.tc_variant(1)  # the other form: the same launch
         t_raw = timed(lambda: ctx.internal_tc(h, None, y_tc, nrhs=R, want_e=False))
         ctx.tc_variant(0)
         d_raw = float(torch.linalg.vector_norm(y_tc - y_mv) / torch.linalg.vector_norm(y_mv))
