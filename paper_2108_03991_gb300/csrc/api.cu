@@ -143,6 +143,7 @@ int aim_gemv_select(aim_ctx* c, int kind) {
   for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);  // they hold the old launches
   c->graphs.clear();
   c->gplan = p;
+  c->gplan_user = kind != 0;
   // the paired launch holds the autotuned shape: another choice runs e = Z h after j's GEMV
   c->z_after = kind != 0 && c->z_tuned == 3 ? 2 : c->z_tuned;
   return BEM_OK;
@@ -152,6 +153,7 @@ int aim_gemv_plan(aim_ctx* c, int kind, int ctas_per_sm, int split, int unroll) 
   BEM_TRY(check_ctx(c, "aim_gemv_plan"));
   BEM_CUDA(cudaDeviceSynchronize());
   BEM_TRY(set_gemv_shape(c, kind, ctas_per_sm, split, unroll));
+  c->gplan_user = true;
   for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);  // they hold the old launches
   c->graphs.clear();
   if (c->z_tuned == 3) c->z_after = 2;  // the paired launch holds the autotuned shape

@@ -283,6 +283,7 @@ struct aim_ctx {
   bem::GemvPlan gplan64;  // FP64 products
   bem::GemvPlan gbg32, gbg64;  // e = Z h beside the AIM chain in the system matvec (few CTAs)
   bem::GemvPlan gpair;         // j = h - C h and e = Z h as one task list (both precisions)
+  bool gplan_user = false;     // gplan is a caller's choice (aim_gemv_select, aim_gemv_plan)
   bem::GemvPlan gm16;          // tasks of 16 rows (more than four right-hand sides: k_gemv_m8)
   bem::GemvPlan gmr;           // several right-hand sides: task list of 16-row tasks (k_gemv_mr)
   bem::GemvPlan gplan_auto;    // the autotuner's FP32 choice

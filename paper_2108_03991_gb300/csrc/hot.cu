@@ -1648,9 +1648,9 @@ int internal(aim_ctx* c, const void* hv, void* ev, void* heqv, int nrhs, cudaStr
   PrecBuf<R>& b = buf<R>(c);
   const GemvPlan& gp = sizeof(R) == 4 ? c->gplan : c->gplan64;
   if constexpr (sizeof(R) == 4) {
-    // more than four right-hand sides: eight at a time (k_gemv_m8). Six bars of 240-1,920 edges, Z and
-    // C (us): 337 -> 117 at 16, 2,719 -> 858 at 128; one bar of 2,016 163 -> 42, 1,315 -> 268
-    if (nrhs > 4 && c->gm16.ntasks > 0 && !(ev && c->zsp_on)) {
+    // more than four right-hand sides: eight at a time (k_gemv_m8), unless the caller pinned a launch
+    // form. Six bars of 240-1,920 edges, Z and C (us): 337 -> 117 at 16, 2,719 -> 858 at 128; one bar of 2,016 163 -> 42, 1,315 -> 268
+    if (nrhs > 4 && c->gm16.ntasks > 0 && !c->gplan_user && !(ev && c->zsp_on)) {
       const V* h = (const V*)hv;
       for (int g = 0; g < nrhs; g += 16 * 65535) {  // gridDim.y
         const int n = std::min(16 * 65535, nrhs - g);

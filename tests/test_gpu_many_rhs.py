@@ -50,3 +50,21 @@ def test_blocks(ctx, nrhs):
     xd = torch.from_numpy(x.astype(np.complex64).ravel()).cuda()
     y = api.blockdiag_gemv(sizes, A, xd, torch.empty_like(xd), nrhs).cpu().numpy().reshape(nrhs, N)
     assert np.all(np.linalg.norm(y - ref, axis=1) <= 1e-5 * np.linalg.norm(ref, axis=1))
+
+
+def test_pinned_form(ctx):
+    """A launch form that the caller chose holds for every count: each group of four gives the bits
+    of a call with that group alone; select(0) gives the eights back."""
+    h = torch.from_numpy(synth.rand_cvec(9 * ctx.ne, 70).astype(np.complex64)).cuda()
+    free = ctx.internal(h, nrhs=9)
+    ctx.gemv_plan(0, 6, 2, 4)
+    try:
+        e, q = ctx.internal(h, nrhs=9)
+        for r, n in ((0, 4), (4, 4), (8, 1)):
+            sl = slice(r * ctx.ne, (r + n) * ctx.ne)
+            e1, q1 = ctx.internal(h[sl].contiguous(), nrhs=n)
+            assert torch.equal(e[sl], e1) and torch.equal(q[sl], q1)
+    finally:
+        ctx.gemv_select(0)
+    for out, ref in zip(ctx.internal(h, nrhs=9), free):
+        assert torch.equal(out, ref)
