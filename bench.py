@@ -786,7 +786,7 @@ def main():
             # columns of K_s + I_x/2), h gathered, the permuted rows written and read, e written
             zb = sp["bytes_c32"] + 4 * 8 * ctx.ne
             zsp = {"kernels": "k_zsp_rows (rows of K_s + I_x/2) + k_zsp_solve (banded L_s^-1, "
-                              "one warp per ring)",
+                              "one CTA per ring)",
                    "bytes": zb, "ms": zsp_ms, "achieved": zb / (zsp_ms * 1e-3) / 1e9,
                    "unit": "GB/s", "frac": zb / (zsp_ms * 1e-3) / 1e9 / hbm,
                    "half_bandwidth": sp["band"], "setup_check": sp["check"],
