@@ -283,6 +283,7 @@ template int run_gemv_mr<double>(const GemvPlan&, const double2*, const double2*
 // warp meet in a reduce-scatter (62 shuffles instead of 320), which leaves row k and right-hand side r
 // of the tile in lane 8 k + r. y_r = A x_r for r < nrhs.
 constexpr int kM8 = 8;
+constexpr int kM8Max = 16 * 65535;  // right-hand sides per launch (gridDim.y takes pairs of eights)
 __device__ __forceinline__ void gemv_m8_task(const GemvTask& t, const float2* __restrict__ A,
                                              const float2* __restrict__ x, float2* __restrict__ y,
                                              int64_t vstride, int nrhs, int rg) {
@@ -819,8 +820,13 @@ static int launch_blk(const BlkTab<CAP>& tab, unsigned ntask, const typename C2<
   if (nrhs == 1) {
     k_gemv_blk<R, CAP><<<ntask, 128, 0, s>>>(tab, A, x, y);
   } else if (sizeof(R) == 4 && nrhs > 4) {
-    if constexpr (sizeof(R) == 4)
-      k_gemv_blk_m8<CAP><<<dim3(ntask, (nrhs + 15) / 16), nrhs > kM8 ? 256 : 128, 0, s>>>(tab, A, x, y, vs, nrhs);
+    if constexpr (sizeof(R) == 4) {
+      for (int64_t g = 0; g < nrhs; g += kM8Max) {
+        const int n = (int)std::min<int64_t>(kM8Max, nrhs - g);
+        k_gemv_blk_m8<CAP><<<dim3(ntask, (n + 15) / 16), n > kM8 ? 256 : 128, 0, s>>>(tab, A, x + g * vs, y + g * vs,
+                                                                                      vs, n);
+      }
+    }
   } else {
     for (int r0 = 0; r0 < nrhs; r0 += 4) {
       const int64_t o = r0 * vs;
@@ -1652,9 +1658,9 @@ int internal(aim_ctx* c, const void* hv, void* ev, void* heqv, int nrhs, cudaStr
     // form. Six bars of 240-1,920 edges, Z and C (us): 337 -> 117 at 16, 2,719 -> 858 at 128; one bar of 2,016 163 -> 42, 1,315 -> 268
     if (nrhs > 4 && c->gm16.ntasks > 0 && !c->gplan_user && !(ev && c->zsp_on)) {
       const V* h = (const V*)hv;
-      for (int g = 0; g < nrhs; g += 16 * 65535) {  // gridDim.y
-        const int n = std::min(16 * 65535, nrhs - g);
-        const int64_t o = (int64_t)g * c->ne;
+      for (int64_t g = 0; g < nrhs; g += kM8Max) {
+        const int n = (int)std::min<int64_t>(kM8Max, nrhs - g);
+        const int64_t o = g * c->ne;
         V *e = ev ? (V*)ev + o : nullptr, *q = heqv ? (V*)heqv + o : nullptr;
         k_gemv_m8<<<dim3(c->gm16.ntasks, (n + 15) / 16, ev && heqv ? 2 : 1), n > kM8 ? 256 : 128, 0, s>>>(
             c->gm16.tasks, ev ? b.Z : b.C, b.C, h + o, ev ? e : q, q, c->ne, n);

@@ -68,3 +68,21 @@ def test_pinned_form(ctx):
         ctx.gemv_select(0)
     for out, ref in zip(ctx.internal(h, nrhs=9), free):
         assert torch.equal(out, ref)
+
+
+def test_blocks_beyond_one_grid(ctx):
+    """More right-hand sides than the pairs of eights of one launch (65,535 along the grid's y): the
+    vectors on both sides of the cut and the last ones, against NumPy."""
+    sizes, nrhs = [1, 2], 16 * 65535 + 5
+    blocks = synth.rand_blocks(sizes, 8)
+    x = torch.randn(nrhs * 3, dtype=torch.complex64, device="cuda")
+    A = torch.from_numpy(api.pack_blocks(blocks, np.complex64)).cuda()
+    y = api.blockdiag_gemv(sizes, A, x, torch.full_like(x, float("nan")), nrhs).view(nrhs, 3)
+    x = x.view(nrhs, 3).to(torch.complex128)
+    ref = torch.empty_like(x)
+    for o, B in zip((0, 1), blocks):
+        k = B.shape[0]
+        ref[:, o:o + k] = x[:, o:o + k] @ torch.from_numpy(B).to(x).T
+    # per vector: |y - ref| <= 1e-5 |A| |x|
+    d = (y - ref).norm(dim=1)
+    assert bool((d <= 1e-5 * max(np.linalg.norm(B) for B in blocks) * x.norm(dim=1)).all())
