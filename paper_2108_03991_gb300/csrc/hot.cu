@@ -1653,31 +1653,34 @@ int internal(aim_ctx* c, const void* hv, void* ev, void* heqv, int nrhs, cudaStr
   typedef typename C2<R>::T V;
   PrecBuf<R>& b = buf<R>(c);
   const GemvPlan& gp = sizeof(R) == 4 ? c->gplan : c->gplan64;
+  const V* h = (const V*)hv;
+  V *e = (V*)ev, *heq = (V*)heqv;
+  if (e && c->zsp_on) {  // e = Z_s h, the sparse internal operator, as many vectors as its scratch takes
+    for (int64_t r = 0; r < nrhs; r += kMaxBatch)
+      BEM_TRY(zsp_apply<R>(c, h + r * c->ne, e + r * c->ne, (int)std::min<int64_t>(kMaxBatch, nrhs - r), c->ne, c->ne,
+                           s));
+    if (!heq) return BEM_OK;
+    e = nullptr;
+  }
   if constexpr (sizeof(R) == 4) {
     // more than four right-hand sides: eight at a time (k_gemv_m8), unless the caller pinned a launch
     // form. Six bars of 240-1,920 edges, Z and C (us): 337 -> 117 at 16, 2,719 -> 858 at 128; one bar of 2,016 163 -> 42, 1,315 -> 268
-    if (nrhs > 4 && c->gm16.ntasks > 0 && !c->gplan_user && !(ev && c->zsp_on)) {
-      const V* h = (const V*)hv;
+    if (nrhs > 4 && c->gm16.ntasks > 0 && !c->gplan_user) {
       for (int64_t g = 0; g < nrhs; g += kM8Max) {
         const int n = (int)std::min<int64_t>(kM8Max, nrhs - g);
         const int64_t o = g * c->ne;
-        V *e = ev ? (V*)ev + o : nullptr, *q = heqv ? (V*)heqv + o : nullptr;
-        k_gemv_m8<<<dim3(c->gm16.ntasks, (n + 15) / 16, ev && heqv ? 2 : 1), n > kM8 ? 256 : 128, 0, s>>>(
-            c->gm16.tasks, ev ? b.Z : b.C, b.C, h + o, ev ? e : q, q, c->ne, n);
+        V *eg = e ? e + o : nullptr, *qg = heq ? heq + o : nullptr;
+        k_gemv_m8<<<dim3(c->gm16.ntasks, (n + 15) / 16, eg && qg ? 2 : 1), n > kM8 ? 256 : 128, 0, s>>>(
+            c->gm16.tasks, eg ? b.Z : b.C, b.C, h + o, eg ? eg : qg, qg, c->ne, n);
       }
       BEM_CUDA(cudaGetLastError());
       return BEM_OK;
     }
   }
-  if (!ev) {
-  } else if (c->zsp_on) {  // e = Z_s h, the sparse internal operator
-    BEM_TRY(zsp_apply<R>(c, (const V*)hv, (V*)ev, nrhs, c->ne, c->ne, s));
-  } else if (nrhs == 1 && heqv && c->z_after == 3 && c->gpair.ntasks > 0) {  // the matvec's pair
-    return run_gemv_pair<R>(c->gpair, b.C, b.Z, (const V*)hv, (V*)heqv, (V*)ev, nullptr, s);
-  } else {
-    BEM_TRY(run_gemv_plan<R>(gp, b.Z, (const V*)hv, (V*)ev, nrhs, c->ne, nullptr, s));
-  }
-  if (heqv) BEM_TRY(run_gemv_plan<R>(gp, b.C, (const V*)hv, (V*)heqv, nrhs, c->ne, nullptr, s));
+  if (e && nrhs == 1 && heq && c->z_after == 3 && c->gpair.ntasks > 0)  // the matvec's pair
+    return run_gemv_pair<R>(c->gpair, b.C, b.Z, h, heq, e, nullptr, s);
+  if (e) BEM_TRY(run_gemv_plan<R>(gp, b.Z, h, e, nrhs, c->ne, nullptr, s));
+  if (heq) BEM_TRY(run_gemv_plan<R>(gp, b.C, h, heq, nrhs, c->ne, nullptr, s));
   return BEM_OK;
 }
 template int internal<float>(aim_ctx*, const void*, void*, void*, int, cudaStream_t);

@@ -86,3 +86,32 @@ def test_blocks_beyond_one_grid(ctx):
     # per vector: |y - ref| <= 1e-5 |A| |x|
     d = (y - ref).norm(dim=1)
     assert bool((d <= 1e-5 * max(np.linalg.norm(B) for B in blocks) * x.norm(dim=1)).all())
+
+
+@pytest.fixture(scope="module")
+def rings():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    c = api.Context(*synth.srr_array_config(2, 2))
+    assert c.sparse_internal["on"]
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("prec", [api.BEM_C32, api.BEM_C64])
+@pytest.mark.parametrize("nrhs", [4, 5, 8, 9, 16])
+def test_internal_sparse(rings, nrhs, prec):
+    """More vectors than the sparse internal operator takes at once, e and h_eq, either and both: e has
+    the bits of a call with that vector alone, h_eq is the FP64 product's (C32 1e-5, C64 1e-12)."""
+    h = torch.from_numpy(synth.rand_cvec(nrhs * rings.ne, 60 + nrhs)).to(api.cdtype(prec)).cuda()
+    e, q = rings.internal(h, nrhs=nrhs, prec=prec)
+    e1, _ = rings.internal(h, nrhs=nrhs, prec=prec, want_heq=False)
+    _, q1 = rings.internal(h, nrhs=nrhs, prec=prec, want_e=False)
+    assert torch.equal(e, e1) and torch.equal(q, q1)
+    for r in range(nrhs):
+        sl = slice(r * rings.ne, (r + 1) * rings.ne)
+        hr = h[sl].contiguous()
+        assert torch.equal(e[sl], rings.internal(hr, prec=prec, want_heq=False)[0])
+        ref = rings.internal(hr.to(torch.complex128), prec=api.BEM_C64, want_e=False)[1]
+        assert float((q[sl] - ref).norm()) <= (1e-5 if prec == api.BEM_C32 else 1e-12) * float(ref.norm())
+    assert not rings.internal_sparse(True)["wait_timed_out"]
