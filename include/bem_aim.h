@@ -116,7 +116,8 @@ const char* bem_last_error(void);
  * (-1: none), [42]=1 if one of its products had a bounded wait time out (that product's e is
  * invalid; reading it synchronises the device), [43]=calls of aim_internal_tc, [44]=1 if one
  * of its products had a bounded wait time out, 0 if none did, -1 before its first call (reading
- * it synchronises the device). Writes min(n, 45) entries. */
+ * it synchronises the device); [45] bit r: FP64 system products of r vectors take the dense Z
+ * although the sparse internal operator is on. Writes min(n, 46) entries. */
 int aim_info(const aim_ctx* ctx, int64_t* info, int n);
 
 /* Sparse internal operator at high frequency (Sec. III-A, third item of the internal problem:
@@ -130,9 +131,10 @@ int aim_info(const aim_ctx* ctx, int64_t* info, int n);
  * at most 256, and Z_s h must match the dense Z h to 1e-8 at set-up (FP64, one probe vector).
  * Then e = Z_s h = -(1/(j k0 eps_rc)) L_s^{-1}(K_s + I_x/2) h replaces e = Z h in aim_matvec,
  * internal_apply and bem_solve (C = Y_eq Z stays dense), and is on after aim_setup. on = 0
- * selects the dense Z again, on = 1 the sparse form (BEM_EINVAL when none was built). The FP64
- * system products (aim_matvec, aim_matvec_batch, bem_solve's residuals) of few objects take the
- * dense Z also then: where it was the faster one at set-up and the two agreed to 1e-13.
+ * selects the dense Z again, on = 1 the sparse form (BEM_EINVAL when none was built). Until a
+ * call of this function chooses, the FP64 system products (aim_matvec, aim_matvec_batch,
+ * bem_solve's residuals) of r vectors take the dense Z where it was the faster one at set-up
+ * and the two agreed to 1e-13 (aim_info entry 45); on = 1 selects Z_s for them too.
  * Synchronises the device; captured matvec graphs are rebuilt on next use. */
 int aim_internal_sparse(aim_ctx* ctx, int on);
 

@@ -297,8 +297,8 @@ class Context:
         self._read_info()
 
     def _read_info(self):
-        info = (C.c_int64 * 45)()
-        _check(lib().aim_info(self.h, info, 45))
+        info = (C.c_int64 * 46)()
+        _check(lib().aim_info(self.h, info, 46))
         self.info = list(info)
         self.ne, self.nt, self.nobj = info[0], info[1], info[2]
         self.n = self.ne + self.nt
@@ -325,7 +325,9 @@ class Context:
         self.sparse_internal = {"setup_s": info[36] * 1e-6, "objects": info[37], "on": bool(info[38]),
                                 "band": info[39], "bytes_c32": info[40],
                                 "check": None if info[41] < 0 else info[41] * 1e-15,
-                                "wait_timed_out": bool(info[42])}
+                                "wait_timed_out": bool(info[42]),
+                                # vectors per product whose FP64 system product is dense all the same
+                                "fp64_dense": [r for r in range(1, 32) if info[45] >> r & 1]}
         # many right-hand sides on the tensor cores (aim_internal_tc): calls, and whether a
         # bounded wait timed out (None before the first call)
         self.tensor_core = {"calls": info[43], "wait_timed_out": None if info[44] < 0 else bool(info[44])}

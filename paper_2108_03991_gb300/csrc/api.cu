@@ -124,6 +124,7 @@ int aim_info(const aim_ctx* c, int64_t* info, int n) {
   int64_t tv[2];
   tc_stats(c, tv);
   for (int i = 43; i < n && i < 45; ++i) info[i] = tv[i - 43];
+  if (n > 45) info[45] = c->zsp_on && !c->zsp_pin ? c->zsp64_dense : 0;
   return BEM_OK;
 }
 
@@ -491,7 +492,7 @@ int aim_internal_sparse(aim_ctx* c, int on) {
   BEM_CUDA(cudaDeviceSynchronize());
   for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);  // they hold the old launches
   c->graphs.clear();
-  c->zsp_on = on != 0;
+  c->zsp_on = c->zsp_pin = on != 0;
   return BEM_OK;
 }
 

@@ -381,8 +381,8 @@ struct aim_ctx {
   // qualifies (zsp_ready), used for e = Z h while zsp_on
   void* zsp = nullptr;
   bool zsp_ready = false, zsp_on = false;
-  // FP64 time of Z_s h and of the dense Z h (ms, one vector; 0: not the same product to rounding)
-  float zsp64_ms[2] = {0, 0};
+  bool zsp_pin = false;      // the sparse form is a caller's choice (aim_internal_sparse)
+  unsigned zsp64_dense = 0;  // bit r: FP64 system products of r vectors take the dense Z (zsp_time)
   // many right-hand sides through Z and C on the tensor cores (zgemm_tc.cu), made on first use
   void* tc = nullptr;
   // form of the row kernels (aim_rows_variant): 0 near sums four-deep with a one-entry tail,
@@ -496,10 +496,11 @@ void zsp_stats(const aim_ctx* c, int64_t* out);
 template <typename R>
 int zsp_apply(aim_ctx* c, const typename C2<R>::T* h, typename C2<R>::T* e, int nrhs, int64_t hs,
               int64_t es, cudaStream_t s);
+// after zsp_check and the GEMV tuners: zsp64_dense
+int zsp_time(aim_ctx* c);
 // whether the system matvec of nrhs vectors takes e = Z_s h (else the dense Z)
 template <typename R> inline bool zsp_used(const aim_ctx* c, int nrhs) {
-  if (!c->zsp_on) return false;
-  return sizeof(R) == 4 || c->zsp64_ms[0] == 0.f || nrhs * c->zsp64_ms[1] >= c->zsp64_ms[0];
+  return c->zsp_on && (sizeof(R) == 4 || c->zsp_pin || !(c->zsp64_dense >> nrhs & 1));
 }
 // many right-hand sides through the FP32 Z and C on the tensor cores (zgemm_tc.cu)
 int internal_tc(aim_ctx* c, const float2* h, float2* e, float2* heq, int nrhs, cudaStream_t s);

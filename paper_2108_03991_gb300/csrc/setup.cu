@@ -1589,6 +1589,9 @@ int setup_device(aim_ctx* c) {
   BEM_TRY(tune_matvec_schedule(c));
   c->setup_ms[9] = wall_ms() - tst;
   c->zsp_on = zsp;
+  tst = wall_ms();
+  BEM_TRY(zsp_time(c));
+  c->setup_ms[10] += wall_ms() - tst;
   return BEM_OK;
 }
 

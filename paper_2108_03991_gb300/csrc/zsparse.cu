@@ -542,6 +542,7 @@ void free_zsp(aim_ctx* c) {
   c->zsp = nullptr;
   c->zsp_ready = false;
   c->zsp_on = false;
+  c->zsp64_dense = 0;
 }
 
 int zsp_prepare(aim_ctx* c, const double* d_verts, const int32_t* d_tris, const double* d_cen) {
@@ -766,27 +767,46 @@ int zsp_check(aim_ctx* c) {
     return BEM_OK;
   }
   c->zsp_on = true;
-  // FP64: a ring's substitutions are bound by the FP64 rate of the one SM they run on, the dense
-  // product by the whole GPU's, so few objects are faster dense (4 rings of 912 edges 35 us against
-  // 413, 36 rings 282 / 453, 256 rings 2,000 / 979). The system matvec takes the faster one where both
-  // are the same product to rounding.
-  if (worst <= kZspSame) {
-    cudaEvent_t ev[3];
-    for (cudaEvent_t& q : ev) BEM_CUDA(cudaEventCreate(&q));
-    cudaEventRecord(ev[0], 0);
-    rc = zsp_apply<double>(c, h, e1, 1, ne, ne, 0);
-    cudaEventRecord(ev[1], 0);
-    if (rc == BEM_OK) rc = run_gemv_plan<double>(c->gplan64, c->f64.Z, h, e2, 1, ne, nullptr, 0);
-    cudaEventRecord(ev[2], 0);
-    cudaError_t sync = cudaEventSynchronize(ev[2]);
-    if (rc == BEM_OK && sync == cudaSuccess) {
-      cudaEventElapsedTime(&c->zsp64_ms[0], ev[0], ev[1]);
-      cudaEventElapsedTime(&c->zsp64_ms[1], ev[1], ev[2]);
+  return BEM_OK;
+}
+
+// FP64: an object's substitutions are bound by the FP64 rate of the one SM they run on, the dense
+// product by the whole GPU's, so few objects are faster dense (4 rings of 912 edges 35 us against 413,
+// 36 rings 282 / 453, 256 rings 2,000 / 979). For every number of vectors of the system products both
+// forms are timed (best of three launches after a first one); the dense one is taken where it is the
+// faster, both are the same product to rounding, and no caller chose the sparse form.
+int zsp_time(aim_ctx* c) {
+  Zsp* z = static_cast<Zsp*>(c->zsp);
+  if (!z || !c->zsp_on || !(z->check <= kZspSame)) return BEM_OK;
+  const int ne = c->ne;
+  double2* h = nullptr;
+  BEM_CUDA(cudaMalloc(&h, 2 * (size_t)kMaxBatch * ne * sizeof(double2)));
+  std::unique_ptr<void, decltype(&cudaFree)> hold(h, &cudaFree);
+  double2* e = h + (size_t)kMaxBatch * ne;
+  k_zsp_probe<<<(kMaxBatch * ne + 255) / 256, 256>>>(h, kMaxBatch * ne);
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  int rc = BEM_OK;
+  cudaError_t err = cudaEventCreate(&ev[0]);
+  if (err == cudaSuccess) err = cudaEventCreate(&ev[1]);
+  for (int r = 1; r <= kMaxBatch && rc == BEM_OK && err == cudaSuccess; ++r) {
+    float best[2] = {1e30f, 1e30f};
+    for (int k = 0; k < 8 && rc == BEM_OK && err == cudaSuccess; ++k) {  // in turn: sparse, dense
+      cudaEventRecord(ev[0], 0);
+      if (k % 2 == 0) rc = zsp_apply<double>(c, h, e, r, ne, ne, 0);
+      else if (r > 1 && c->gmr.ntasks > 0) rc = run_gemv_mr<double>(c->gmr, c->f64.Z, h, e, r, ne, nullptr, 0);
+      else rc = run_gemv_plan<double>(c->gplan64, c->f64.Z, h, e, r, ne, nullptr, 0);
+      cudaEventRecord(ev[1], 0);
+      err = cudaEventSynchronize(ev[1]);
+      float ms = 1e30f;
+      if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, ev[0], ev[1]);
+      if (k >= 2) best[k % 2] = std::min(best[k % 2], ms);
     }
-    for (cudaEvent_t& q : ev) cudaEventDestroy(q);
-    BEM_TRY(rc);
-    BEM_CUDA(sync);
+    if (best[1] < best[0]) c->zsp64_dense |= 1u << r;
   }
+  for (cudaEvent_t q : ev)
+    if (q) cudaEventDestroy(q);
+  BEM_TRY(rc);
+  BEM_CUDA(err);
   return BEM_OK;
 }
 

@@ -48,3 +48,30 @@ def test_sparse_against_dense(make, lo, hi):
                 assert np.linalg.norm(s - d) <= tol * np.linalg.norm(d)
     assert not ctx.internal_sparse(True)["wait_timed_out"]
     ctx.close()
+
+
+def test_explicit_choice_holds():
+    """FP64 system products of one to four vectors on two rings: dense after set-up (two rings are
+    bound by two SMs' FP64 rate otherwise), sparse once a caller chose the sparse form, which the
+    status reports and the bits show (both forms agree to 1e-12, not to the last bit)."""
+    ctx = api.Context(*rings(60, 2))
+    n0 = ctx.sparse_internal["fp64_dense"]
+    assert ctx.sparse_internal["on"] and 1 in n0
+
+    def products():
+        out = []
+        for r in range(1, 5):
+            x = torch.from_numpy(synth.rand_cvec(r * ctx.n, 40 + r)).cuda()
+            y = ctx.matvec(x, prec=api.BEM_C64) if r == 1 else ctx.matvec_batch(x, prec=api.BEM_C64)
+            out.append(y.view(r, ctx.n)[:, :ctx.ne].clone())
+        return out
+    auto = products()
+    assert ctx.internal_sparse(True)["fp64_dense"] == []
+    sparse = products()
+    assert ctx.internal_sparse(False)["fp64_dense"] == []
+    dense = products()
+    for r, (a, s, d) in enumerate(zip(auto, sparse, dense), 1):
+        assert torch.equal(a, d if r in n0 else s)
+        assert not torch.equal(s, d) and float((s - d).norm()) <= 1e-12 * float(d.norm())
+    assert not ctx.internal_sparse(True)["wait_timed_out"]
+    ctx.close()
