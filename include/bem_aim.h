@@ -117,7 +117,8 @@ const char* bem_last_error(void);
  * invalid; reading it synchronises the device), [43]=calls of aim_internal_tc, [44]=1 if one
  * of its products had a bounded wait time out, 0 if none did, -1 before its first call (reading
  * it synchronises the device); [45] bit r: FP64 system products of r vectors take the dense Z
- * although the sparse internal operator is on. Writes min(n, 46) entries. */
+ * although the sparse internal operator is on; [46]=the check of entry 41 for the FP32 Z_s h
+ * against the FP64 Z h, in units of 1e-12 (-1: none). Writes min(n, 47) entries. */
 int aim_info(const aim_ctx* ctx, int64_t* info, int n);
 
 /* Sparse internal operator at high frequency (Sec. III-A, third item of the internal problem:
@@ -128,7 +129,8 @@ int aim_info(const aim_ctx* ctx, int64_t* info, int n);
  * radii, nearest of the 2 x 2 triangle pairs); the kept pattern is ordered by reverse
  * Cuthill-McKee and L_s factorised as a band without pivoting (FP64, then rounded for the FP32
  * path); the band and the kept rows must be below half the dense Z's bytes, the half-bandwidth
- * at most 256, and Z_s h must match the dense Z h to 1e-8 at set-up (FP64, one probe vector).
+ * at most 192, and Z_s h must match the dense FP64 Z h at set-up (one probe vector): to 1e-8 in
+ * FP64 and to 1e-5 in FP32.
  * Then e = Z_s h = -(1/(j k0 eps_rc)) L_s^{-1}(K_s + I_x/2) h replaces e = Z h in aim_matvec,
  * internal_apply and bem_solve (C = Y_eq Z stays dense), and is on after aim_setup. on = 0
  * selects the dense Z again, on = 1 the sparse form (BEM_EINVAL when none was built). Until a

@@ -297,8 +297,8 @@ class Context:
         self._read_info()
 
     def _read_info(self):
-        info = (C.c_int64 * 46)()
-        _check(lib().aim_info(self.h, info, 46))
+        info = (C.c_int64 * 47)()
+        _check(lib().aim_info(self.h, info, 47))
         self.info = list(info)
         self.ne, self.nt, self.nobj = info[0], info[1], info[2]
         self.n = self.ne + self.nt
@@ -325,6 +325,7 @@ class Context:
         self.sparse_internal = {"setup_s": info[36] * 1e-6, "objects": info[37], "on": bool(info[38]),
                                 "band": info[39], "bytes_c32": info[40],
                                 "check": None if info[41] < 0 else info[41] * 1e-15,
+                                "check_c32": None if info[46] < 0 else info[46] * 1e-12,
                                 "wait_timed_out": bool(info[42]),
                                 # vectors per product whose FP64 system product is dense all the same
                                 "fp64_dense": [r for r in range(1, 32) if info[45] >> r & 1]}

@@ -14,8 +14,8 @@
 // inverse, a block's columns streamed into shared memory by one bulk copy while earlier blocks
 // are worked on). C = Y_eq Z stays dense, so j = h - C h is unchanged and e = Z_s h, needed only
 // by the I_x e term of the system matvec, runs beside it. The sparse form is used when every object
-// qualifies (band and rows below half the dense bytes, b <= 256) and a set-up check of Z_s h
-// against the dense Z h (FP64, one probe vector) stays below 1e-8.
+// qualifies (band and rows below half the dense bytes, b <= 192) and a set-up check of Z_s h
+// against the dense FP64 Z h (one probe vector) stays below 1e-8, and below 1e-5 in FP32.
 #include <algorithm>
 #include <cmath>
 #include <complex>
@@ -40,6 +40,7 @@ constexpr int kZspW32 = 32, kZspW64 = 16, kZspW64s = 8;
 constexpr int kZspRing = 256;        // second accumulator, a ring over rows (>= 192 + 32)
 constexpr int kZspStages = 3;        // slabs in flight (2 where shared memory leaves no room)
 constexpr double kZspCheck = 1e-8;   // set-up check of Z_s h against Z h
+constexpr double kZspCheck32 = 1e-5;  // that of the FP32 Z_s h, against the FP64 Z h
 constexpr double kZspSame = 1e-13;  // below it Z_s h and Z h are the same product to FP64 rounding
 constexpr double kTwoPi = 6.283185307179586476925;
 
@@ -65,7 +66,7 @@ struct Zsp {
   int* d_err = nullptr;    // set by a product whose bounded wait timed out
   float2* v32 = nullptr;   // [kMaxBatch][ne] rows of K_s + I_x/2 h, permuted (product scratch)
   double2* v64 = nullptr;
-  double check = -1;  // max over objects of |Z_s h - Z h| / |Z h| at set-up
+  double check = -1, check32 = -1;  // max over objects of |Z_s h - Z h| / |Z h| at set-up, FP64 and FP32 Z_s
   ~Zsp() {
     if (W) cudaFree(W);
   }
@@ -723,34 +724,8 @@ __global__ void k_zsp_probe(double2* h, int n) {
   h[i] = make_double2((double)(v >> 40) / 8388608.0 - 1.0, (double)((v >> 8) & 0xFFFFFF) / 8388608.0 - 1.0);
 }
 
-// Z_s h against the dense Z h (FP64) for one probe vector; the sparse form is kept when every
-// object agrees to kZspCheck
-int zsp_check(aim_ctx* c) {
-  Zsp* z = static_cast<Zsp*>(c->zsp);
-  if (!z) return BEM_OK;
-  const int ne = c->ne;
-  double2 *h = nullptr, *e1 = nullptr, *e2 = nullptr;
-  BEM_CUDA(cudaMalloc(&h, 3 * (size_t)ne * sizeof(double2)));
-  std::unique_ptr<void, decltype(&cudaFree)> hold(h, &cudaFree);
-  e1 = h + ne;
-  e2 = h + 2 * (size_t)ne;
-  k_zsp_probe<<<(ne + 255) / 256, 256>>>(h, ne);
-  c->zsp_ready = true;
-  int rc = zsp_apply<double>(c, h, e1, 1, ne, ne, 0);
-  if (rc == BEM_OK) rc = run_gemv_plan<double>(c->gplan64, c->f64.Z, h, e2, 1, ne, nullptr, 0);
-  if (rc != BEM_OK) {
-    free_zsp(c);
-    return rc;
-  }
-  std::vector<double2> a(ne), d(ne);
-  int err = 0;
-  BEM_CUDA(cudaMemcpy(&err, z->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (err) {  // a bounded wait of the product timed out: keep the dense form
-    free_zsp(c);
-    return BEM_OK;
-  }
-  BEM_CUDA(cudaMemcpy(a.data(), e1, ne * sizeof(double2), cudaMemcpyDeviceToHost));
-  BEM_CUDA(cudaMemcpy(d.data(), e2, ne * sizeof(double2), cudaMemcpyDeviceToHost));
+// largest over the objects of |a - d| / |d|
+template <typename V> static double zsp_worst(const Zsp* z, const std::vector<V>& a, const std::vector<double2>& d) {
   double worst = 0;
   for (const ZspObj& o : z->obj) {
     double num = 0, den = 0;
@@ -759,10 +734,48 @@ int zsp_check(aim_ctx* c) {
       num += dx * dx + dy * dy;
       den += d[r].x * d[r].x + d[r].y * d[r].y;
     }
-    worst = std::max(worst, den > 0 ? std::sqrt(num / den) : (num > 0 ? 1.0 : 0.0));
+    const double q = num == 0 ? 0.0 : std::sqrt(num / den);
+    if (!(q <= worst) && worst == worst) worst = q;  // a NaN stays
   }
-  z->check = worst;
-  if (!(worst <= kZspCheck)) {
+  return worst;
+}
+
+// Z_s h against the dense Z h (FP64) for one probe vector, whose entries FP32 holds exactly; the
+// sparse form is kept when every object agrees to kZspCheck in FP64 and to kZspCheck32 in FP32,
+// which has tables of its own (wider blocks, whose inverses are rounded)
+int zsp_check(aim_ctx* c) {
+  Zsp* z = static_cast<Zsp*>(c->zsp);
+  if (!z) return BEM_OK;
+  const int ne = c->ne;
+  double2* h = nullptr;
+  BEM_CUDA(cudaMalloc(&h, 4 * (size_t)ne * sizeof(double2)));
+  std::unique_ptr<void, decltype(&cudaFree)> hold(h, &cudaFree);
+  double2 *e1 = h + ne, *e2 = h + 2 * (size_t)ne;
+  float2 *h32 = reinterpret_cast<float2*>(h + 3 * (size_t)ne), *e32 = h32 + ne;
+  k_zsp_probe<<<(ne + 255) / 256, 256>>>(h, ne);
+  k_round_kv<<<(ne + 255) / 256, 256>>>(h, h32, ne);
+  c->zsp_ready = true;
+  int rc = zsp_apply<double>(c, h, e1, 1, ne, ne, 0);
+  if (rc == BEM_OK) rc = zsp_apply<float>(c, h32, e32, 1, ne, ne, 0);
+  if (rc == BEM_OK) rc = run_gemv_plan<double>(c->gplan64, c->f64.Z, h, e2, 1, ne, nullptr, 0);
+  if (rc != BEM_OK) {
+    free_zsp(c);
+    return rc;
+  }
+  std::vector<double2> a(ne), d(ne);
+  std::vector<float2> f(ne);
+  int err = 0;
+  BEM_CUDA(cudaMemcpy(&err, z->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  if (err) {  // a bounded wait of the product timed out: keep the dense form
+    free_zsp(c);
+    return BEM_OK;
+  }
+  BEM_CUDA(cudaMemcpy(a.data(), e1, ne * sizeof(double2), cudaMemcpyDeviceToHost));
+  BEM_CUDA(cudaMemcpy(f.data(), e32, ne * sizeof(float2), cudaMemcpyDeviceToHost));
+  BEM_CUDA(cudaMemcpy(d.data(), e2, ne * sizeof(double2), cudaMemcpyDeviceToHost));
+  z->check = zsp_worst(z, a, d);
+  z->check32 = zsp_worst(z, f, d);
+  if (!(z->check <= kZspCheck && z->check32 <= kZspCheck32)) {
     free_zsp(c);
     return BEM_OK;
   }
@@ -819,6 +832,7 @@ void zsp_stats(const aim_ctx* c, int64_t* out) {
     out[3] = 0;
     out[4] = -1;
     out[5] = 0;
+    out[6] = -1;
     return;
   }
   out[0] = (int64_t)z->obj.size();
@@ -826,6 +840,7 @@ void zsp_stats(const aim_ctx* c, int64_t* out) {
   out[2] = z->bmax;
   out[3] = 2 * z->nband * 8 + (int64_t)c->ne * 8 + z->nnz * 12;
   out[4] = (int64_t)(z->check * 1e15);
+  out[6] = (int64_t)(z->check32 * 1e12);
   int err = 0;  // set by a product whose bounded wait timed out
   if (cudaMemcpy(&err, z->d_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) err = -1;
   out[5] = err;

@@ -75,3 +75,31 @@ def test_explicit_choice_holds():
         assert not torch.equal(s, d) and float((s - d).norm()) <= 1e-12 * float(d.norm())
     assert not ctx.internal_sparse(True)["wait_timed_out"]
     ctx.close()
+
+
+def _probe(n):
+    """The set-up check's probe vector: a hash of the index, 24 bits a part."""
+    v = np.arange(n, dtype=np.uint64) * np.uint64(0x9E3779B97F4A7C15) + np.uint64(0xD1B54A32D192ED03)
+    v ^= v >> np.uint64(31)
+    v *= np.uint64(0xBF58476D1CE4E5B9)
+    v ^= v >> np.uint64(29)
+    part = lambda b: b.astype(np.float64) / 2.0 ** 23 - 1.0  # noqa: E731
+    return part(v >> np.uint64(40)) + 1j * part((v >> np.uint64(8)) & np.uint64(0xFFFFFF))
+
+
+@pytest.mark.parametrize("make", [thin_bar, lambda: rings(80, 3)])
+def test_fp32_form_is_checked(make):
+    """The set-up check covers the FP32 tables: the status reports their error against the FP64 dense
+    Z h, below 1e-5, and it is the one measured here (to a percent: it is rounded to 1e-12)."""
+    mesh, grid, freq = make()
+    ctx = api.Context(mesh, grid, freq)
+    check = ctx.sparse_internal["check_c32"]
+    assert ctx.sparse_internal["on"] and check is not None and 0 < check < 1e-5
+    h = torch.from_numpy(_probe(ctx.ne)).cuda()
+    e = ctx.internal(h.to(torch.complex64), want_heq=False)[0].cpu().numpy()
+    ctx.internal_sparse(False)
+    d = ctx.internal(h, prec=api.BEM_C64, want_heq=False)[0].cpu().numpy()
+    worst = max(np.linalg.norm(a - b) / np.linalg.norm(b)
+                for a, b in zip(np.split(e, mesh.nobj), np.split(d, mesh.nobj)))
+    assert abs(worst - check) <= 0.01 * worst
+    ctx.close()
