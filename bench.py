@@ -519,7 +519,7 @@ def bar_array_section(args, api, synth, torch, np, dev):
 
 def tensor_core_section(ctx, api, synth, torch, np, dev, hbm, reps=10):
     """h_eq = C h for R right-hand sides at once (C = Y_eq Z, complex FP32): the tensor-core
-    product (one pass over C per 128 right-hand sides, scaled FP16 hi and lo parts) against the
+    product (one pass over C per 128 right-hand sides, three BF16 parts a value) against the
     block GEMV (one pass per 4), both through the library; the two agree to FP32 rounding. Per
     R: ms per product, C's bytes over that time, and the complex flops 8 sum n_i^2 R over it."""
     ZY = ctx.zy_bytes_c32 // 2

@@ -225,19 +225,19 @@ int internal_apply(aim_ctx* ctx, const void* h, void* e, void* heq, int nrhs, in
  * Sec. II-C) for r < nrhs, complex FP32 (interleaved re, im), the right-hand sides stored one
  * after another, each N_E long, in the conductor-contiguous order of aim_matvec. Every block is
  * streamed from device memory once per 128 right-hand sides: each complex block product is one
- * real GEMM (FP16 tensor cores, hi/lo split of both scaled operands, 22 bits, FP32 sums). Always the
- * dense Z, also while the sparse internal operator is on. Either output may be NULL (not both);
+ * real GEMM (BF16 tensor cores, both operands split into three parts that hold an FP32 value's 24
+ * bits at every magnitude above 2^-110, six part products, FP32 sums). Always the dense Z,
+ * also while the sparse internal operator is on. Either output may be NULL (not both);
  * h, e and h_eq must not alias. Asynchronous on `stream`; the first call builds the per-object
- * operand descriptors and the workspace for packed right-hand sides and partial sums (NP sum ld_i
- * FP32 values and up to 0.5 KB NP per unit of work, NP = 2 nrhs rounded up to 32, 64, 128 or 256;
- * it grows and synchronises `stream` when a later call needs more). A bounded wait that times out leaves that product invalid and
- * shows in aim_info[44]. Errors: BEM_EINVAL (bad pointers, nrhs < 1, no FP32 blocks),
+ * operand descriptors and the workspace for packed right-hand sides and partial sums (12 NP bytes
+ * per unknown and up to 0.5 KB NP per unit of work, NP = 2 nrhs rounded up to 32, 64, 128 or 256;
+ * it grows and synchronises `stream` when a later call needs more). A bounded wait that times out
+ * leaves that product invalid and shows in aim_info[44]. Errors: BEM_EINVAL (bad pointers, nrhs < 1, no FP32 blocks),
  * BEM_ENOMEM, BEM_ECUDA (the driver has no tensor-map encoder, or a launch failed). */
 int aim_internal_tc(aim_ctx* ctx, const void* h, void* e, void* heq, int nrhs, void* stream);
 
-/* Form of aim_internal_tc's product, 0 or 1: kept for callers that choose one; the packed
- * right-hand sides now take the bytes of the raw ones, and both select the same launch (the same
- * bits). Errors: BEM_EINVAL. */
+/* Form of aim_internal_tc's product, 0 or 1: kept for callers that choose one; both
+ * select the same launch (the same bits). Errors: BEM_EINVAL. */
 int aim_tc_variant(aim_ctx* ctx, int variant);
 
 /* The grid step H of Eq. AIM_L alone: phi_c = sum_b G_grid(a - b) sigma_c(b) (linear

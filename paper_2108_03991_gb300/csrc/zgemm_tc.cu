@@ -9,35 +9,37 @@
 //   column 2r + 1 = ( Im x_0,  Re x_0,  Im x_1,  Re x_1, ...)   (gives Im y_r),
 // so D = A_real B (M = n, K = 2n, N = 2R) holds y_r as the (re, im) pair of columns 2r, 2r + 1.
 //
-// FP32 accuracy from FP16 tensor cores by the three-product split. Every row of A and every
-// (object, right-hand side) slice of x is scaled by the power of two that brings its largest entry
-// into [2^14, 2^15); then a = a_hi + a_lo with a_hi the nearest FP16 value and a_lo the nearest FP16
-// value of the rest, 22 significant bits (entries below 2^-18 of the largest keep 2^-40 of it), and
-// D = A_hi B_hi + A_hi B_lo + A_lo B_hi in FP32, scaled back exactly. The dropped A_lo B_lo is 2^-22.
-// The split of an FP32 tile into TF32 parts, the form before, has the same 22 bits but twice the bytes
-// in shared memory, twice the MMAs at half their rate, and twice the truncations of the accumulator.
+// FP32 accuracy from BF16 tensor cores by a three-part split: a = a1 + a2 + a3, a1 the leading 8
+// significant bits of the FP32 value (truncated), a2 the nearest BF16 value of the rest, a3 what is
+// left, which BF16 holds exactly: all 24 bits, at every magnitude, since BF16 has FP32's exponents.
+// D = A1 B1 + (A1 B2 + A2 B1 + A2 B2 + A1 B3 + A3 B1) in FP32; the dropped A2 B3 + A3 B2 is below 2^-22.
+// (Two scaled FP16 parts, 22 bits, need half the MMAs, but entries far below the largest of their row
+// or slice lose bits: 5 exponent bits. A column of Z falls by 2^-100 along a bar of 30 skin depths, and
+// a unit vector's product has to return it.) Two TF32 parts take as many MMAs and more shared memory.
 //
-// Layout. B is packed once per call from x into [N][K_tot]: every object's K range starts at a
-// multiple of 32 values and every 32 values of a row are 128 bytes, 32 FP16 hi parts then their 32 lo
-// parts (zeros past the object's 2 n values). A is read in place through one 2-D tensor map per
-// object (inner extent 2n floats, rows n, row pitch 8 ld bytes): TMA fills the K tail and the rows
-// past n with zeros; the landed FP32 tile is turned in place into the same [32 hi | 32 lo] rows.
-// Shared-memory tiles are K-major with the 128-byte swizzle.
+// Layout. B is packed once per call from x into [3 parts][N][K_tot]: every object's K range starts at a
+// multiple of 32 values, and 32 values of a row are 64 bytes (zeros past the object's 2 n values). A is
+// read in place through one 2-D tensor map per object (inner extent 2n floats, rows n, row pitch 8 ld
+// bytes): TMA fills the K tail and the rows past n with zeros; the landed FP32 tile is turned in place
+// into rows of 32 first parts and 32 second parts, its third parts go to a tile beside it. Shared-memory
+// tiles are K-major; rows of 128 bytes (A) have the 128-byte swizzle, rows of 64 bytes (A3, B) the
+// 64-byte one. The parts of B follow each other, so that one MMA multiplies A1 by two or three of them.
 //
-// A product is bound by shared memory (a stage of 32 K values moves 112 KB through it at N = 128: the
-// landing tiles, the conversion, the operands of 6 MMAs) and by the HBM reads of the blocks, so both
+// A product is bound by shared memory (a stage of 32 K values moves 168 KB through it at N = 128: the
+// landing tiles, the conversion, the operands of 10 MMAs) and by the HBM reads of the blocks, so both
 // matrices go in one launch of persistent CTAs and the K loops of the tiles are cut into units that
-// load them evenly (tc_units). Z and C together, packing included, against one launch per matrix with
-// a CTA per tile in TF32 (us, 64 right-hand sides): six bars of 240-1,920 edges 257 -> 69, one bar of
-// 2,016 263 -> 40, 16 rings of 912 144 -> 72; 128 right-hand sides 539 -> 100, 446 -> 56, 262 -> 104;
-// 144 rings (HBM-bound) 395 at 1, 467 at 64. Error against 64 bits on the rings 6.6e-6 -> 2.2e-6.
+// load them evenly (tc_units). Z and C together, packing included (us, 64 right-hand sides): six bars of
+// 240-1,920 edges 79, one bar of 2,016 46, 16 rings of 912 91 (257, 263, 144 with one launch per matrix
+// and a CTA per tile in TF32; 69, 40, 72 with two FP16 parts); 16 right-hand sides 61, 36, 68; 128 of
+// them 121, 64, 132 (539, 446, 262; 100, 56, 105); 144 rings 414 at 1 (HBM-bound), 637 at 64 (395, 468).
+// Error against 64 bits on the bars 4.5e-7, on the rings 2.2e-6 (TF32 6.6e-6), the accumulator's.
 // Every wait is bounded: on a timeout the CTA records an error (err[0], kept across products)
 // and raises the launch's abort flag (err[1], cleared before each launch), waits (with a short
 // limit) for its own MMAs and copies in flight, frees its TMEM and leaves; the other CTAs see
 // the flag in their waits, or before they start, and leave too. The results are then invalid.
 #include <cuda.h>
 #include <cudaTypedefs.h>
-#include <cuda_fp16.h>
+#include <cuda_bf16.h>
 
 #include <algorithm>
 
@@ -52,14 +54,15 @@ constexpr int kTcK = 32;        // floats of K per stage: one 128-byte swizzle r
 // group waits on its loads and its proxy fence while the others work, and never waits for a phase
 // of its stage that is two ahead.
 template <int NP> struct TcShape;
-template <> struct TcShape<32> { static constexpr int S = 8, G = 32; };
-template <> struct TcShape<64> { static constexpr int S = 7, G = 32; };
-template <> struct TcShape<128> { static constexpr int S = 6, G = 64; };
-template <> struct TcShape<256> { static constexpr int S = 4, G = 64; };
+template <> struct TcShape<32> { static constexpr int S = 7, G = 64; };
+template <> struct TcShape<64> { static constexpr int S = 6, G = 64; };
+template <> struct TcShape<128> { static constexpr int S = 4, G = 128; };
+template <> struct TcShape<256> { static constexpr int S = 3, G = 128; };
 constexpr int kTcEpi = 128;  // threads that read the accumulators, one row of a tile each
 template <int NP> constexpr int tc_threads() { return kTcEpi + 64 + TcShape<NP>::S * TcShape<NP>::G; }
 constexpr int kTcMaxRhs = 128;  // N = 2R <= 256 per launch
-constexpr uint32_t kTcAtile = kTcM * kTcK * 4;  // 16 KB
+constexpr uint32_t kTcAtile = kTcM * kTcK * 4;  // 16 KB: FP32, then the first and second parts
+constexpr uint32_t kTcA3 = kTcM * kTcK * 2;     // 8 KB: the third parts
 
 struct TcUnit {  // stages [k0, k1) of one 128-row tile of one block of Z (mat 0) or C (mat 1)
   int32_t obj, row0, mat, k0, k1;
@@ -79,10 +82,16 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
-// instruction descriptor of kind::f16: D in FP32 (bits 4-5 = 1), A and B FP16 (bits 7-9 and 10-12 =
-// 0), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
-__host__ __device__ constexpr uint32_t f16_idesc(int M, int N) {
-  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// the same with rows of 64 bytes, 8-row groups 512 bytes apart, layout type 4 (64-byte swizzle: the
+// 16-byte vector v of row r at v ^ ((r >> 1) & 3))
+__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)4 << 61);
+}
+// instruction descriptor of kind::f16: D in FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9 and 10-12 =
+// 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
+__host__ __device__ constexpr uint32_t bf16_idesc(int M, int N) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, int x, int y, uint64_t* bar) {
@@ -107,7 +116,7 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-__device__ __forceinline__ void tc_mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
+__device__ __forceinline__ void tc_mma_bf16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
                                             uint32_t accumulate) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -137,23 +146,17 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
-// exponent shift that brings a slice's largest magnitude m into [2^14, 2^15); 0 for a zero slice
-__device__ __forceinline__ int tc_shift(float m) {
-  if (!(m > 0.f)) return 0;
-  const int e = (int)(__float_as_uint(m) >> 23) - 127;  // floor(log2 m); -127 below the normal range
-  return min(126, 14 - e);
-}
-__device__ __forceinline__ float tc_pow2(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
-__device__ __forceinline__ uint32_t h2(float a, float b) {
-  const __half2 v = __floats2half2_rn(a, b);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
-// hi and lo parts of two scaled values
-__device__ __forceinline__ void tc_halves(float a, float b, uint32_t* hi, uint32_t* lo) {
-  const __half2 h = __floats2half2_rn(a, b);
-  const float2 f = __half22float2(h);
-  *hi = *reinterpret_cast<const uint32_t*>(&h);
-  *lo = h2(a - f.x, b - f.y);
+// the three BF16 parts of two values, packed
+__device__ __forceinline__ void tc_split(float a, float b, uint32_t* p1, uint32_t* p2, uint32_t* p3) {
+  const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
+  *p1 = __byte_perm(ua, ub, 0x7632);
+  const float ra = a - __uint_as_float(ua & 0xFFFF0000u), rb = b - __uint_as_float(ub & 0xFFFF0000u);
+  const __nv_bfloat162 m = __floats2bfloat162_rn(ra, rb);
+  const uint32_t um = *reinterpret_cast<const uint32_t*>(&m);
+  *p2 = um;
+  const __nv_bfloat162 l =
+      __floats2bfloat162_rn(ra - __uint_as_float(um << 16), rb - __uint_as_float(um & 0xFFFF0000u));
+  *p3 = *reinterpret_cast<const uint32_t*>(&l);
 }
 
 // Bounded wait on an mbarrier phase that also gives up as soon as any CTA of the launch has
@@ -176,93 +179,54 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, const in
   return false;
 }
 
-// exponent shift of every row of a block-diagonal matrix (set-up of the first product): one warp per row
-__global__ void __launch_bounds__(256) k_tc_rowshift(const TcObj* __restrict__ objs, const int64_t* __restrict__ off,
-                                                     const float2* __restrict__ A, int32_t* __restrict__ sh) {
-  const TcObj o = objs[blockIdx.y];
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= o.n) return;
-  const float2* a = A + off[blockIdx.y] + (int64_t)row * ((o.n + 3) & ~3);
-  float m = 0.f;
-  for (int k = lane; k < o.n; k += 32) m = fmaxf(m, fmaxf(fabsf(a[k].x), fabsf(a[k].y)));
-#pragma unroll
-  for (int q = 16; q > 0; q >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, q));
-  if (lane == 0) sh[o.xoff + row] = tc_shift(m);
-}
-
-// (re, im) 2^-sh, in two factors of normal range
-__device__ __forceinline__ float2 tc_unscale(float re, float im, int sh) {
-  const int e1 = -sh >> 1;
-  const float f1 = tc_pow2(e1), f2 = tc_pow2(-sh - e1);
-  return make_float2(re * f1 * f2, im * f1 * f2);
-}
-
-// B from x: rows 2r and 2r + 1 of right-hand side r < R (zero rows up to NP), one CTA per object and
-// right-hand side: the slice's largest entry, then its 2 n values as FP16 hi and lo parts, zeros up
-// to the object's padded length
+// B from x: rows 2r and 2r + 1 of right-hand side r < R (zero rows up to NP) of the three parts (pstride
+// words apart), one CTA per object and right-hand side: the slice's 2 n values, zeros up to the object's
+// padded length; a word holds two values
 __global__ void __launch_bounds__(256) k_tc_pack(const float2* __restrict__ x, int64_t vstride, int R,
                                                  const TcObj* __restrict__ objs, int64_t ktot,
-                                                 uint32_t* __restrict__ b, int32_t* __restrict__ shb) {
+                                                 uint32_t* __restrict__ b, int64_t pstride) {
   const TcObj o = objs[blockIdx.x];
   const int r = blockIdx.y;
   const float2* xs = x + r * vstride + o.xoff;
-  float m = 0.f;
-  if (r < R)
-    for (int k = threadIdx.x; k < o.n; k += 256) m = fmaxf(m, fmaxf(fabsf(xs[k].x), fabsf(xs[k].y)));
-  __shared__ float red[8];
-#pragma unroll
-  for (int q = 16; q > 0; q >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, q));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < 8; ++q) m = fmaxf(m, red[q]);
-  const int sh = tc_shift(m);
-  const float s = tc_pow2(sh);
-  if (threadIdx.x == 0) shb[blockIdx.x * (int64_t)kTcMaxRhs + r] = sh;
-  // in units of 4 bytes (two FP16 values): slot u of 32-value chunk q is hi at 32 q + u, lo 16 further
-  uint32_t* b0 = b + 2 * r * ktot + o.koff;
-  uint32_t* b1 = b0 + ktot;
+  uint32_t* p = b + 2 * r * ktot + o.koff;
   for (int k = threadIdx.x; k < (o.n + 15 & ~15); k += 256) {
-    float2 v = make_float2(0.f, 0.f);
-    if (r < R && k < o.n) v = make_float2(xs[k].x * s, xs[k].y * s);
-    uint32_t hi, lo;
-    const int64_t at = 32 * (int64_t)(k >> 4) + (k & 15);
-    tc_halves(v.x, -v.y, &hi, &lo);
-    b0[at] = hi;
-    b0[at + 16] = lo;
-    tc_halves(v.y, v.x, &hi, &lo);
-    b1[at] = hi;
-    b1[at + 16] = lo;
+    const float2 v = r < R && k < o.n ? xs[k] : make_float2(0.f, 0.f);
+    tc_split(v.x, -v.y, p + k, p + pstride + k, p + 2 * pstride + k);
+    tc_split(v.y, v.x, p + ktot + k, p + pstride + ktot + k, p + 2 * pstride + ktot + k);
   }
 }
 
-// shared memory of one CTA: S stages of [A | B], each tile 1024-byte aligned, then the barriers, the
-// TMEM slot
+// shared memory of one CTA: S stages of [A | A3 | B1 | B2 | B3], each tile 1024-byte aligned, then the
+// barriers, the TMEM slot
 template <int NP> struct TcSmem {
   static constexpr int S = TcShape<NP>::S;
-  static constexpr uint32_t kStage = kTcAtile + NP * kTcK * 4;
+  static constexpr uint32_t kB = kTcAtile + kTcA3, kBp = NP * kTcK * 2;  // kBp: bytes of one part of B
+  static constexpr uint32_t kStage = kB + 3 * kBp;
+  static constexpr uint32_t kTx = kStage - kTcA3;  // bytes landing per stage
   static constexpr uint32_t kBars = S * kStage;
   static constexpr uint32_t kBytes = kBars + 8 * (3 * S + 5) + 16 + 1024;  // + alignment slack
 };
 
-// one row of a landed FP32 tile (128 bytes, its 16-byte vectors swizzled by the row) scaled and turned
-// in place into 32 FP16 hi parts and 32 lo parts
-__device__ __forceinline__ void tc_convert_row(uint8_t* tile, int row, float s) {
+// one row of a landed FP32 tile (128 bytes, its 16-byte vectors swizzled by the row) turned in place
+// into 32 first parts and 32 second parts, the third parts to the tile after it
+__device__ __forceinline__ void tc_convert_row(uint8_t* tile, int row) {
   float4* a = reinterpret_cast<float4*>(tile + row * 128);
-  const int x = row & 7;
+  uint4* a3 = reinterpret_cast<uint4*>(tile + kTcAtile + row * 64);
+  const int x = row & 7, x3 = row >> 1 & 3;
   float4 v[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) v[c] = a[c ^ x];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const float4 p = v[2 * j], q = v[2 * j + 1];
-    uint4 hi, lo;
-    tc_halves(p.x * s, p.y * s, &hi.x, &lo.x);
-    tc_halves(p.z * s, p.w * s, &hi.y, &lo.y);
-    tc_halves(q.x * s, q.y * s, &hi.z, &lo.z);
-    tc_halves(q.z * s, q.w * s, &hi.w, &lo.w);
-    reinterpret_cast<uint4*>(a)[j ^ x] = hi;
-    reinterpret_cast<uint4*>(a)[(4 + j) ^ x] = lo;
+    uint4 h, m, l;
+    tc_split(p.x, p.y, &h.x, &m.x, &l.x);
+    tc_split(p.z, p.w, &h.y, &m.y, &l.y);
+    tc_split(q.x, q.y, &h.z, &m.z, &l.z);
+    tc_split(q.z, q.w, &h.w, &m.w, &l.w);
+    reinterpret_cast<uint4*>(a)[j ^ x] = h;
+    reinterpret_cast<uint4*>(a)[(4 + j) ^ x] = m;
+    a3[j ^ x3] = l;
   }
 }
 
@@ -270,25 +234,26 @@ __device__ __forceinline__ void tc_convert_row(uint8_t* tile, int row, float s) 
 // is the stages [k0, k1) of the K loop of one 128-row tile of one block of one of the two matrices.
 // Warps 0-3 read the accumulators, warp 4 issues the TMA loads, warp 5 the MMAs, the others convert the
 // landed tiles; stages pass from one to the next through mbarriers and run on across units, and
-// (NP <= 128) the accumulators are double, so a unit's start-up and its epilogue cost nothing. A_hi
-// B_hi is accumulated apart from the cross terms (NP columns each): the tensor core truncates every
-// accumulation, and the cross terms, 2^-11 as large, would triple the number of truncations of the
-// large sum. The parts of a tile cut into several units go to a workspace, which k_tc_reduce sums (the
+// (NP <= 128) the accumulators are double, so a unit's start-up and its epilogue cost nothing. A1 B1
+// is accumulated apart from the other five terms (NP columns, 2 NP where TMEM has them): the tensor core
+// truncates every accumulation, and those terms, 2^-7 as large, would make the truncations of the large
+// sum six times as many. The parts of a tile cut into several units go to a workspace, which k_tc_reduce sums (the
 // unit that finishes last, four warps on one SM, took 50 us for it).
 template <int NP>
 __global__ void __launch_bounds__(tc_threads<NP>(), 1)
     k_zgemm_tc(const __grid_constant__ CUtensorMap mb, const CUtensorMap* __restrict__ mz,
                const CUtensorMap* __restrict__ mc, const TcUnit* __restrict__ units, int nunit,
                const int32_t* __restrict__ nst, const TcObj* __restrict__ objs,
-               const int32_t* __restrict__ shz, const int32_t* __restrict__ shc,
-               const int32_t* __restrict__ shb, float2* __restrict__ yz, float2* __restrict__ yc,
-               int64_t vstride, int R, float4* __restrict__ part, int* err) {
+               float2* __restrict__ yz, float2* __restrict__ yc, int64_t vstride, int R,
+               float4* __restrict__ part, int* err) {
   typedef TcSmem<NP> L;
   constexpr int S = L::S, kG = TcShape<NP>::G;
-  constexpr int NACC = NP <= 128 ? 2 : 1;          // accumulator pairs in TMEM
-  constexpr uint32_t kCols = NACC * 2 * NP;
-  constexpr uint32_t kTx = L::kStage;              // bytes landing per stage
-  constexpr uint32_t kIdesc = f16_idesc(kTcM, NP);
+  constexpr int NACC = NP <= 128 ? 2 : 1;          // sets of accumulators in TMEM
+  constexpr uint32_t kAcc = (NP <= 64 ? 3 : 2) * NP;  // columns of one: A1 B1, then the other terms
+  constexpr uint32_t kCols = NP == 32 ? 256 : 512;
+  static_assert(NACC * kAcc <= kCols, "TMEM columns");
+  constexpr uint32_t kIdesc = bf16_idesc(kTcM, NP), kIdesc2 = bf16_idesc(kTcM, NP <= 128 ? 2 * NP : NP),
+                     kIdesc3 = bf16_idesc(kTcM, NP <= 64 ? 3 * NP : NP);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* full = reinterpret_cast<uint64_t*>(base + L::kBars);  // [S] the stage's loads have landed
@@ -327,7 +292,7 @@ __global__ void __launch_bounds__(tc_threads<NP>(), 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot;  // pair q: columns 2 NP q + [0, NP) A_hi B_hi, + [NP, 2 NP) the cross terms
+  const uint32_t tmem = *tslot;  // set q: columns kAcc q + [0, NP) A1 B1, then the other terms
 
   int issued = 0;  // producer: stages whose loads are issued
   bool ok = true;
@@ -348,13 +313,17 @@ __global__ void __launch_bounds__(tc_threads<NP>(), 1)
       tc_fence_after();
       const int row = u.row0 + trow, cend = min(NP, (2 * R + 15) & ~15);
       float2* y = u.mat ? yc : yz;
-      const int sa = row < o.n ? (u.mat ? shc : shz)[o.xoff + row] : 0;
-      const int32_t* sb = shb + u.obj * (int64_t)kTcMaxRhs;
-      const uint32_t tl = tmem + 2 * NP * q + ((uint32_t)(warp * 32) << 16);
+      const uint32_t tl = tmem + kAcc * q + ((uint32_t)(warp * 32) << 16);
       for (int c0 = 0; c0 < cend; c0 += 16) {
         float v[16], w[16];
         tc_ld16(tl + c0, v);
         tc_ld16(tl + NP + c0, w);
+        if constexpr (kAcc > 2 * NP) {
+          float w2[16];
+          tc_ld16(tl + 2 * NP + c0, w2);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) w[k] += w2[k];
+        }
 #pragma unroll
         for (int k = 0; k < 16; ++k) v[k] += w[k];
         if (u.parts > 1) {
@@ -365,7 +334,7 @@ __global__ void __launch_bounds__(tc_threads<NP>(), 1)
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
             const int r = c0 / 2 + k;
-            if (r < R) y[r * vstride + o.xoff + row] = tc_unscale(v[2 * k], v[2 * k + 1], sa + __ldg(sb + r));
+            if (r < R) y[r * vstride + o.xoff + row] = make_float2(v[2 * k], v[2 * k + 1]);
           }
         }
       }
@@ -388,10 +357,11 @@ __global__ void __launch_bounds__(tc_threads<NP>(), 1)
             break;
           }
           uint8_t* st = base + slot * L::kStage;
-          const int kx = (int)(o.koff + (int64_t)kc * kTcK);
-          mbar_arrive_tx(&full[slot], kTx);
+          const int kx = (int)(o.koff + (int64_t)kc * (kTcK / 2));  // in words of two values
+          mbar_arrive_tx(&full[slot], L::kTx);
           tma_load_2d(st, mA, kc * kTcK, u.row0, &full[slot]);
-          tma_load_2d(st + kTcAtile, &mb, kx, 0, &full[slot]);
+#pragma unroll
+          for (int p = 0; p < 3; ++p) tma_load_2d(st + L::kB + p * L::kBp, &mb, kx, p * NP, &full[slot]);
           ++issued;
           if (++slot == S) {
             slot = 0;
@@ -410,22 +380,35 @@ __global__ void __launch_bounds__(tc_threads<NP>(), 1)
           break;
         }
         tc_fence_after();
-        const uint32_t d = tmem + 2 * NP * q;
+        const uint32_t d = tmem + kAcc * q;
         for (int kc = k0; kc < k1; ++kc) {
           if (!tc_wait(&full[slot], ph, abort_flag, kTcSpin) || !tc_wait(&conv[slot], ph, abort_flag, kTcSpin)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t sa = smem_u32(base + slot * L::kStage), sb = sa + kTcAtile;
+          const uint32_t sa = smem_u32(base + slot * L::kStage), sb = sa + L::kB;
 #pragma unroll
-          for (int k = 0; k < kTcK / 16; ++k) {  // 16 FP16 = 32 bytes of K per instruction; lo 64 bytes on
-            const uint64_t ah = sw128_desc(sa + 32 * k), al = sw128_desc(sa + 64 + 32 * k);
-            const uint64_t bh = sw128_desc(sb + 32 * k), bl = sw128_desc(sb + 64 + 32 * k);
+          for (int k = 0; k < kTcK / 16; ++k) {  // 16 BF16 = 32 bytes of K per instruction
+            const uint64_t a1 = sw128_desc(sa + 32 * k), a2 = sw128_desc(sa + 64 + 32 * k);
+            const uint64_t a3 = sw64_desc(sa + kTcAtile + 32 * k), b1 = sw64_desc(sb + 32 * k);
+            const uint64_t b2 = sw64_desc(sb + L::kBp + 32 * k), b3 = sw64_desc(sb + 2 * L::kBp + 32 * k);
             const uint32_t acc = (kc > k0 || k > 0) ? 1u : 0u;
-            tc_mma_f16(d, ah, bh, kIdesc, acc);
-            tc_mma_f16(d + NP, al, bh, kIdesc, acc);
-            tc_mma_f16(d + NP, ah, bl, kIdesc, 1u);
+            if constexpr (NP <= 64) {
+              tc_mma_bf16(d, a1, b1, kIdesc3, acc);        // A1 [B1 B2 B3]
+              tc_mma_bf16(d + NP, a2, b1, kIdesc2, 1u);    // A2 [B1 B2], onto A1 B2 and A1 B3
+            } else {
+              if constexpr (NP == 128) {
+                tc_mma_bf16(d, a1, b1, kIdesc2, acc);      // A1 [B1 B2]
+              } else {
+                tc_mma_bf16(d, a1, b1, kIdesc, acc);
+                tc_mma_bf16(d + NP, a1, b2, kIdesc, acc);
+              }
+              tc_mma_bf16(d + NP, a2, b1, kIdesc, 1u);
+              tc_mma_bf16(d + NP, a2, b2, kIdesc, 1u);
+              tc_mma_bf16(d + NP, a1, b3, kIdesc, 1u);
+            }
+            tc_mma_bf16(d + NP, a3, b1, kIdesc, 1u);
           }
           tc_commit(&empty[slot]);
           if (++slot == S) {
@@ -440,26 +423,8 @@ __global__ void __launch_bounds__(tc_threads<NP>(), 1)
     // a group converts the stages of its slot, a thread the rows t, t + kG, ... of each
     constexpr int kRows = kTcM / kG;
     const int t = (tid - 192) % kG, slot = (tid - 192) / kG, total = nst[blockIdx.x];
-    int ph = 0, ui = blockIdx.x, first = 0, last = 0;  // stages [first, last) belong to unit ui
-    float sc[kRows];
+    int ph = 0;
     for (int i = slot; i < total; i += S, ph ^= 1) {
-      bool moved = last == 0;
-      if (moved) last = units[ui].k1 - units[ui].k0;
-      while (i >= last) {
-        ui += gridDim.x;
-        first = last;
-        last = first + units[ui].k1 - units[ui].k0;
-        moved = true;
-      }
-      if (moved) {
-        const TcUnit u = units[ui];
-        const TcObj o = objs[u.obj];
-#pragma unroll
-        for (int k = 0; k < kRows; ++k) {
-          const int row = u.row0 + t + k * kG;
-          sc[k] = row < o.n ? tc_pow2((u.mat ? shc : shz)[o.xoff + row]) : 0.f;
-        }
-      }
       ok = tc_wait(&full[slot], ph, abort_flag, kTcSpin);
       if (!__all_sync(0xffffffffu, ok)) {
         ok = false;
@@ -467,7 +432,7 @@ __global__ void __launch_bounds__(tc_threads<NP>(), 1)
       }
       uint8_t* st = base + slot * L::kStage;
 #pragma unroll
-      for (int k = 0; k < kRows; ++k) tc_convert_row(st, t + k * kG, sc[k]);
+      for (int k = 0; k < kRows; ++k) tc_convert_row(st, t + k * kG);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(&conv[slot]);
@@ -499,10 +464,8 @@ __global__ void __launch_bounds__(tc_threads<NP>(), 1)
 // y of the tiles cut along K: the sum of their parts in order; one CTA per tile and 16 columns
 template <int NP>
 __global__ void __launch_bounds__(kTcM) k_tc_reduce(const TcUnit* __restrict__ tiles, const TcObj* __restrict__ objs,
-                                                    const int32_t* __restrict__ shz, const int32_t* __restrict__ shc,
-                                                    const int32_t* __restrict__ shb, const float4* __restrict__ part,
-                                                    float2* __restrict__ yz, float2* __restrict__ yc,
-                                                    int64_t vstride, int R) {
+                                                    const float4* __restrict__ part, float2* __restrict__ yz,
+                                                    float2* __restrict__ yc, int64_t vstride, int R) {
   const TcUnit u = tiles[blockIdx.x];
   const TcObj o = objs[u.obj];
   const int row = u.row0 + threadIdx.x, c0 = 16 * blockIdx.y;
@@ -520,14 +483,12 @@ __global__ void __launch_bounds__(kTcM) k_tc_reduce(const TcUnit* __restrict__ t
       a[c] = make_float4(a[c].x + t.x, a[c].y + t.y, a[c].z + t.z, a[c].w + t.w);
     }
   }
-  const int sa = (u.mat ? shc : shz)[o.xoff + row];
-  const int32_t* sb = shb + u.obj * (int64_t)kTcMaxRhs;
   float2* y = (u.mat ? yc : yz) + o.xoff + row;
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const int r = c0 / 2 + 2 * c;
-    if (r < R) y[r * vstride] = tc_unscale(a[c].x, a[c].y, sa + __ldg(sb + r));
-    if (r + 1 < R) y[(r + 1) * vstride] = tc_unscale(a[c].z, a[c].w, sa + __ldg(sb + r + 1));
+    if (r < R) y[r * vstride] = make_float2(a[c].x, a[c].y);
+    if (r + 1 < R) y[(r + 1) * vstride] = make_float2(a[c].z, a[c].w);
   }
 }
 
@@ -547,9 +508,7 @@ struct TcState {
   } units[3];                 // Z alone, C alone, both
   TcObj* objs = nullptr;
   int64_t ktot = 0;           // 32-bit words per row of the packed B
-  uint32_t* b = nullptr;      // packed B, [np_cap][ktot]
-  int32_t *shz = nullptr, *shc = nullptr;  // [ne] exponent shifts of the rows of Z and C
-  int32_t* shb = nullptr;     // [nobj][kTcMaxRhs] of the right-hand sides' slices
+  uint32_t* b = nullptr;      // packed B, [3][NP][ktot]
   float4* part = nullptr;     // partial sums of tiles cut along K
   int np_cap = 0;
   int* err = nullptr;         // [2]: a wait timed out in some product (sticky); this launch gave up
@@ -558,8 +517,7 @@ struct TcState {
     for (Units& u : units)
       for (void* p : {(void*)u.d, (void*)u.nst, (void*)u.cut})
         if (p) cudaFree(p);
-    for (void* p : {(void*)mz, (void*)mc, (void*)objs, (void*)b, (void*)shz, (void*)shc, (void*)shb, (void*)part,
-                    (void*)err})
+    for (void* p : {(void*)mz, (void*)mc, (void*)objs, (void*)b, (void*)part, (void*)err})
       if (p) cudaFree(p);
   }
 };
@@ -577,20 +535,21 @@ static TcEncode tc_encoder() {
   return fn;
 }
 
-// 2-D FP32 tensor map, inner extent `inner` floats, `rows` rows `pitch` bytes apart, box of
-// 32 floats x box_rows, 128-byte swizzle, zero fill outside
+// 2-D tensor map of 4-byte elements, inner extent `inner` of them, `rows` rows `pitch` bytes apart, box
+// of box_cols (32 or 16: 128 or 64 bytes, swizzled over that width) x box_rows, zero fill outside
 static int tc_map(TcEncode enc, CUtensorMap* m, const void* base, int64_t inner, int64_t rows,
-                  int64_t pitch, int box_rows) {
+                  int64_t pitch, int box_cols, int box_rows) {
   const cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)pitch};
-  const cuuint32_t box[2] = {(cuuint32_t)kTcK, (cuuint32_t)box_rows};
+  const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
   const cuuint32_t es[2] = {1, 1};
   if ((reinterpret_cast<uintptr_t>(base) & 15) || (pitch & 15)) {
     set_error("tensor-core product: operand not 16-byte aligned");
     return BEM_EINVAL;
   }
   const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides,
-                         box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                         box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                         box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_error("tensor-core product: cuTensorMapEncodeTiled failed (%d)", (int)r);
@@ -674,13 +633,13 @@ static int tc_prepare(aim_ctx* c, TcState** out) {
   for (int i = 0, xo = 0; i < c->nobj && rc == BEM_OK; ++i) {
     const int n = c->e1[i] - c->e0[i], ld = c->zld[i];
     objs[i] = TcObj{n, xo, ktot};
-    ktot += 2 * round_up(n, 16);
-    rc = tc_map(enc, &mz[i], c->f32.Z + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcM);
-    if (rc == BEM_OK) rc = tc_map(enc, &mc[i], c->f32.C + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcM);
+    ktot += round_up(n, 16);
+    rc = tc_map(enc, &mz[i], c->f32.Z + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcK, kTcM);
+    if (rc == BEM_OK) rc = tc_map(enc, &mc[i], c->f32.C + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcK, kTcM);
     xo += n;
   }
   if (rc == BEM_OK && ktot > INT32_MAX) {
-    set_error("tensor-core product: more than 2^30 unknowns");
+    set_error("tensor-core product: more than 2^31 unknowns");
     rc = BEM_EINVAL;
   }
   t->ktot = ktot;
@@ -714,27 +673,6 @@ static int tc_prepare(aim_ctx* c, TcState** out) {
   up((void**)&t->objs, objs.data(), objs.size() * sizeof(TcObj));
   const int zero[2] = {0, 0};  // [0]: a wait timed out in some product; [1]: this launch gave up
   up((void**)&t->err, zero, sizeof(zero));
-  // exponent shifts of the matrices' rows
-  int64_t* doff = nullptr;
-  int nmax = 0;
-  for (const TcObj& o : objs) nmax = std::max(nmax, o.n);
-  const std::vector<int32_t> none((size_t)std::max<int64_t>(c->ne, c->nobj * (int64_t)kTcMaxRhs), 0);
-  up((void**)&t->shz, none.data(), (size_t)c->ne * sizeof(int32_t));
-  up((void**)&t->shc, none.data(), (size_t)c->ne * sizeof(int32_t));
-  up((void**)&t->shb, none.data(), (size_t)c->nobj * kTcMaxRhs * sizeof(int32_t));
-  up((void**)&doff, c->zoff.data(), (size_t)c->nobj * sizeof(int64_t));
-  if (rc == BEM_OK && nmax > 0) {
-    for (int o0 = 0; o0 < c->nobj; o0 += 65535) {  // gridDim.y
-      const dim3 g((nmax + 7) / 8, std::min(65535, c->nobj - o0));
-      k_tc_rowshift<<<g, 256>>>(t->objs + o0, doff + o0, c->f32.Z, t->shz);
-      k_tc_rowshift<<<g, 256>>>(t->objs + o0, doff + o0, c->f32.C, t->shc);
-    }
-    if (cudaDeviceSynchronize() != cudaSuccess) {
-      set_error("tensor-core product: %s", cudaGetErrorString(cudaGetLastError()));
-      rc = BEM_ECUDA;
-    }
-  }
-  if (doff) cudaFree(doff);
   if (rc != BEM_OK) {
     delete t;
     return rc;
@@ -753,11 +691,10 @@ static int tc_launch(TcState* t, const CUtensorMap& mb, float2* yz, float2* yc, 
   // per call: the attribute belongs to the current device (cheap next to the product)
   BEM_CUDA(cudaFuncSetAttribute(k_zgemm_tc<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
   BEM_CUDA(cudaMemsetAsync(t->err + 1, 0, sizeof(int), s));
-  k_zgemm_tc<NP><<<q.ctas, tc_threads<NP>(), kSmem, s>>>(mb, t->mz, t->mc, q.d, q.n, q.nst, t->objs, t->shz,
-                                                         t->shc, t->shb, yz, yc, vstride, R, t->part, t->err);
+  k_zgemm_tc<NP><<<q.ctas, tc_threads<NP>(), kSmem, s>>>(mb, t->mz, t->mc, q.d, q.n, q.nst, t->objs, yz, yc,
+                                                         vstride, R, t->part, t->err);
   if (q.ncut > 0)
-    k_tc_reduce<NP><<<dim3(q.ncut, (2 * R + 15) / 16), kTcM, 0, s>>>(q.cut, t->objs, t->shz, t->shc, t->shb, t->part,
-                                                                     yz, yc, vstride, R);
+    k_tc_reduce<NP><<<dim3(q.ncut, (2 * R + 15) / 16), kTcM, 0, s>>>(q.cut, t->objs, t->part, yz, yc, vstride, R);
   BEM_CUDA(cudaGetLastError());
   return BEM_OK;
 }
@@ -779,7 +716,7 @@ int internal_tc(aim_ctx* c, const float2* h, float2* e, float2* heq, int nrhs, c
       t->b = nullptr;
       t->part = nullptr;
       t->np_cap = 0;
-      const size_t bytes = (size_t)NP * t->ktot * sizeof(uint32_t);
+      const size_t bytes = (size_t)3 * NP * t->ktot * sizeof(uint32_t);
       int slots = 0;
       for (const TcState::Units& q : t->units) slots = std::max(slots, q.slots);
       const size_t pbytes = (size_t)slots * kTcM * NP * sizeof(float) + 16;
@@ -789,9 +726,9 @@ int internal_tc(aim_ctx* c, const float2* h, float2* e, float2* heq, int nrhs, c
       }
       t->np_cap = NP;
     }
-    CUtensorMap mb;  // 32 words of a row are one stage
-    BEM_TRY(tc_map(enc, &mb, t->b, t->ktot, NP, t->ktot * (int64_t)sizeof(uint32_t), NP));
-    k_tc_pack<<<dim3(c->nobj, NP / 2), 256, 0, s>>>(h + r0 * ne, ne, R, t->objs, t->ktot, t->b, t->shb);
+    CUtensorMap mb;  // 16 words of a row are one stage
+    BEM_TRY(tc_map(enc, &mb, t->b, t->ktot, 3 * NP, 4 * t->ktot, kTcK / 2, NP));
+    k_tc_pack<<<dim3(c->nobj, NP / 2), 256, 0, s>>>(h + r0 * ne, ne, R, t->objs, t->ktot, t->b, NP * t->ktot);
     BEM_CUDA(cudaGetLastError());
     float2* yz = e ? e + r0 * ne : nullptr;
     float2* yc = heq ? heq + r0 * ne : nullptr;

@@ -54,3 +54,22 @@ def test_units_and_scales(ctx, nrhs):
             d = np.linalg.norm(out[:, a:b] - ref[:, a:b], axis=1)
             assert np.all(d <= 1e-5 * np.linalg.norm(ref[:, a:b], axis=1))
     assert ctx.tensor_core_status()["wait_timed_out"] is False
+
+
+def test_unit_vectors(ctx):
+    """A unit vector (one edge, one port) gives back a column of Z and of C, whose entries fall by tens of
+    binades along a bar: each real and imaginary part within 2^-22 of the FP32 entry (three parts hold its
+    24 bits; two accumulators and their sum round once each). Entries and products below 2^-100 are left
+    out: the third part of one below 2^-110 leaves the normal range of BF16 (and FP32) numbers."""
+    ks = [0, 1, ctx.ne // 3, ctx.ne // 2 + 1, ctx.ne - 1] * 4
+    h = torch.zeros(len(ks), ctx.ne, dtype=torch.complex64, device="cuda")
+    for r, k in enumerate(ks):
+        h[r, k] = 2.0 ** (7 * r - 60)
+    for out, ref in zip(ctx.internal_tc(h.view(-1), nrhs=len(ks)), ctx.internal(h.view(-1), nrhs=len(ks))):
+        out = torch.view_as_real(out).double().view(len(ks), -1)
+        ref = torch.view_as_real(ref).double().view(len(ks), -1)
+        entry = ref / h.abs().amax(dim=1, keepdim=True).double()
+        live = (entry.abs() >= 2.0 ** -100) & (ref.abs() >= 2.0 ** -100)
+        assert bool(((out - ref).abs() <= 2.0 ** -22 * ref.abs())[live].all())
+        assert float(entry.abs()[entry != 0].min() / entry.abs().max()) < 2.0 ** -18
+    assert ctx.tensor_core_status()["wait_timed_out"] is False
