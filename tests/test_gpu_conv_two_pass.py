@@ -76,3 +76,32 @@ def test_small_planes(prec, n):
     for c in range(3):
         assert np.linalg.norm(out[c] - ref[c]) <= (2e-6 if prec == api.BEM_C32 else 1e-12) * np.linalg.norm(ref[c])
     ctx.close()
+
+
+RADICES = [1, 2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16, 18, 20, 24, 25, 27, 30, 32]
+
+
+@pytest.mark.parametrize("n,slab", [((500, 60, 8), True), ((540, 61, 12), True), ((486, 500, 8), True),
+                                    ((520, 90, 16), True), ((61, 540, 12), False), ((520, 90, 17), False),
+                                    ((400, 401, 20), False)])
+def test_lengths_without_two_passes(n, slab):
+    """FP32 grids that the two-pass form does not take: an x or y length that is no product of two radices
+    (the slab passes where nz <= 16 and their slab fits shared memory, else the line passes), or a y-z
+    slab beyond shared memory (line passes). 2e-6 and 1e-5 of the largest value, as the other convolution tests; one component and two."""
+    grid = synth.Grid(np.array([-1.1, -1.1, -1.1]), np.array([0.5, 0.4, 0.5]), np.array(n))
+    freq = 3e13
+    ctx = api.Context(synth.bar_mesh(1.0, 1.0, 1.0, 0.5), grid, freq)
+    P = ctx.padded
+    two = [any(P[a] % r == 0 and P[a] // r in RADICES for r in RADICES) for a in (0, 1)]
+    assert not all(two) or 8 * P[1] * P[2] > 200 * 1024  # else the two-pass form takes it
+    floats2 = P[1] + P[2] + (P[2] // 2 + 1) * (P[1] // 2 + 1) + 2 * n[2] * (P[1] + P[1] // 16 + 1)
+    assert slab == (n[2] <= 16 and 8 * floats2 <= 200 * 1024)
+    s = synth.rand_cvec(2 * ctx.ng, 13).reshape(2, n[2], n[1], n[0])
+    ref = _reference(ctx, grid, freq, n, s)
+    for ncomp in (1, 2):
+        d = torch.from_numpy(s[:ncomp].astype(np.complex64).ravel()).cuda()
+        out = ctx.conv(d, ncomp=ncomp).cpu().numpy().reshape(s[:ncomp].shape)
+        for c in range(ncomp):
+            assert np.linalg.norm(out[c] - ref[c]) <= 2e-6 * np.linalg.norm(ref[c])
+            assert np.abs(out[c] - ref[c]).max() <= 1e-5 * np.abs(ref[c]).max()
+    ctx.close()
