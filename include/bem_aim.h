@@ -216,7 +216,7 @@ int aim_matvec_host(aim_ctx* ctx, int which, const void* x, void* y, int nvec, i
  * (not both): h_eq alone is the one block GEMV of C = Y_eq Z. With one right-hand side, both
  * outputs, the dense Z and the paired matvec schedule (aim_matvec_schedule mode 3), the two
  * products are one launch, as in the system matvec; with the sparse internal operator
- * (aim_internal_sparse) e = Z_s h. */
+ * (aim_internal_sparse) e = Z_s h, four right-hand sides per launch. */
 int internal_apply(aim_ctx* ctx, const void* h, void* e, void* heq, int nrhs, int prec,
                    void* stream);
 
@@ -232,8 +232,9 @@ int internal_apply(aim_ctx* ctx, const void* h, void* e, void* heq, int nrhs, in
  * operand descriptors and the workspace for packed right-hand sides and partial sums (12 NP bytes
  * per unknown and up to 0.5 KB NP per unit of work, NP = 2 nrhs rounded up to 32, 64, 128 or 256;
  * it grows and synchronises `stream` when a later call needs more). A bounded wait that times out
- * leaves that product invalid and shows in aim_info[44]. Errors: BEM_EINVAL (bad pointers, nrhs < 1, no FP32 blocks),
- * BEM_ENOMEM, BEM_ECUDA (the driver has no tensor-map encoder, or a launch failed). */
+ * leaves that product invalid and shows in aim_info[44]. Errors: BEM_EINVAL (bad pointers,
+ * nrhs < 1, no FP32 blocks), BEM_ENOMEM, BEM_ECUDA (the driver has no tensor-map encoder, or a
+ * launch failed). */
 int aim_internal_tc(aim_ctx* ctx, const void* h, void* e, void* heq, int nrhs, void* stream);
 
 /* Form of aim_internal_tc's product, 0 or 1: kept for callers that choose one; both

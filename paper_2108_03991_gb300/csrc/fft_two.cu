@@ -11,8 +11,9 @@
 //               ky (in registers when Pz is a radix, else as two passes over Pz rows), times Ghat, and
 //               back, in place
 //   x inverse : the mirror of the first launch
-// Bound by the workspace's traffic (L2 or HBM) and the shared-memory trips: a value crosses shared
-// memory 2 times per line where the forms before (shuffle stages in a warp, 10 shuffles a value;
+// Bound by the shared-memory pipe at 16 warps per SM (512 x 512 x 8: k_two_yz 66% of its peak, 9% of DRAM's;
+// 100 to 128 registers for radices above 16), on small grids by instruction fetch: a value crosses
+// shared memory 2 times per line where the forms before (shuffle stages in a warp, 10 shuffles a value;
 // radix-8 Stockham passes with a trip per stage; five passes over the whole padded grid where nz > 16;
 // or a whole plane per CTA, which leaves SMs without one) took 5 to 25.
 // Three components (us): 512 x 512 x 8 399 -> 326, 256 x 256 x 8 101 -> 92, 150 x 90 x 21 242 -> 65, 400 x 300 x
@@ -491,7 +492,8 @@ static bool two_args(const aim_ctx* c, TwoArgs* p, size_t* xsm, size_t* ysm) {
   *xsm = (size_t)kTwoRows * p->x.pitch * sizeof(float2);
   const size_t slab = (size_t)(p->zreg ? p->nz : p->Pz) * p->y.pitch * sizeof(float2);
   p->nk = 1;
-  // two kx per CTA where both together leave room for three CTAs per SM
+  // two kx per CTA where both together leave shared memory for three CTAs per SM (registers for four up to
+  // radix 16, for two above)
   if (p->zreg && 2 * slab <= 70 * 1024) p->nk = 2;
   *ysm = p->nk * slab;
   return *xsm <= kTwoSmem && *ysm <= kTwoSmem;

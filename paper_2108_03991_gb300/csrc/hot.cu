@@ -279,7 +279,8 @@ template int run_gemv_mr<double>(const GemvPlan&, const double2*, const double2*
 // columns, so a 16-byte load of the matrix meets 8 vectors and every load of x serves 4 rows; the next
 // vector of each row is in flight while the current one is used. The two groups of 4 warps of a CTA
 // take the same 16 rows and neighbouring eights of right-hand sides (the second group's matrix loads
-// hit L1). Bound by the FP32 pipe (8 flops per entry and right-hand side). The 32 complex partial sums of a
+// hit L1). Bound by the FP32 pipe (8 flops per entry and right-hand side), which is 36% active: 16 warps
+// per SM wait for loads the rest of the time. The 32 complex partial sums of a
 // warp meet in a reduce-scatter (62 shuffles instead of 320), which leaves row k and right-hand side r
 // of the tile in lane 8 k + r. y_r = A x_r for r < nrhs.
 constexpr int kM8 = 8;
@@ -765,9 +766,9 @@ template int run_gemv<double>(const GemvTask*, int, const double2*, const double
 // reads of the argument). The tasks are those of the task-list form, which the set-up's tuner
 // finds the fastest on most structures: small, handed out by the hardware, largest blocks first.
 // A persistent launch over a table of all rows, built and uploaded on each call, was the form
-// before. FP32, one right-hand side: 1,024 blocks of 912 (6.8 GB) 3,445 -> 960 us, 100 of them 543
-// -> 97, 300 of 1-700 629 -> 66, 4 of 120 216 -> 17 us (the host's call); FP64, 100 of 912 1,199 ->
-// 762 us, then at the FP64 rate.
+// before. FP32, one right-hand side, the whole call: 1,024 blocks of 912 (6.8 GB) 3,445 -> 1,065 us (the
+// launch alone 960), 100 of them 543 -> 97, 300 of 1-700 629 -> 66, 4 of 120 216 -> 17 us (the host's
+// call); FP64, 100 of 912 1,199 -> 762 us, then at the FP64 rate.
 template <int CAP> struct BlkTab {
   int nblk;
   uint32_t first[CAP];  // first task of block b

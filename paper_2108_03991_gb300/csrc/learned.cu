@@ -115,9 +115,9 @@ __device__ __forceinline__ void load_halo(const T* __restrict__ in, const Dims& 
 // out[co][p] = act( sum_ci sum_taps w[co][ci][tap] in[ci][p + tap - 1] ) (* mask[co][p] > 0), the sum
 // of an output in the order ci, tap. Weights as [ci][tap][co] (k_prep_w). A thread has four
 // points along x and half of the output channels: per (ci, dz, dy) it reads six values and 3 CO/2
-// weights (broadcast) for 12 CO/2 multiply-adds. Bound by the FP32 pipe: a layer of 16 to 16
-// channels on 35 x 35 x 78 points is 0.66 G multiply-adds (18 us at 36 T/s; about half the pipe is
-// reached, the tiles' staging and ten warps per SM leave the rest). With one point per thread, 16
+// weights (broadcast) for 12 CO/2 multiply-adds. Bound by the FP32 pipe (45% active): a layer of 16 to 16
+// channels on 35 x 35 x 78 points is 0.66 G multiply-adds (18 us at 36 T/s, 39 measured: 0.86 of a wave
+// of CTAs, the shared-memory pipe at 65% of its peak). With one point per thread, 16
 // scalar weight loads for 16 multiply-adds, per-channel staging and the weight gradient's two loads
 // per multiply-add, a forward and backward pass on that grid took 3.13 ms, a host round trip of
 // the input and 14 allocations included; now 0.73 ms.

@@ -1,12 +1,13 @@
 // bem_blockdiag_gemv_noalloc: the block-diagonal GEMV for callers that cannot allocate device
 // memory. The paper has no counterpart; it is a service of this library.
 //
-// Who needs it: bem_blockdiag_gemv builds its row-panel work list in device memory that it
-// allocates (cudaMallocAsync) on every call. Some callers cannot allow that: programs whose
-// device memory is owned entirely by another allocator (a framework's caching allocator that
-// reserved the whole GPU, so a further cudaMalloc fails or fragments it), and real-time loops
-// whose rules forbid any allocation once they are running. This entry point allocates nothing:
-// its work list lives in a fixed device array compiled into the library.
+// Its callers: programs whose device memory is owned entirely by another allocator (a framework's
+// caching allocator that reserved the whole GPU, so a further cudaMalloc fails or fragments it),
+// and real-time loops whose rules forbid any allocation once they are running. This entry point
+// allocates nothing: its work list lives in a fixed device array compiled into the library.
+// bem_blockdiag_gemv allocates nothing either: its table of blocks is a kernel argument, it has no
+// limit on the panels, shares no scratch between calls and can be captured. New callers take that
+// one; this one keeps its limits and refusals for those that rely on them.
 //
 // The scratch: kNoAllocMaxTasks tasks (32 bytes each, 1 MiB) in a file-scope __device__ array.
 // Every GPU that loads the library holds it until the process exits. In host code the array's

@@ -560,8 +560,8 @@ static int tc_map(TcEncode enc, CUtensorMap* m, const void* base, int64_t inner,
 
 // The units of a product over the matrices in `mats` (bit 0 Z, bit 1 C): every tile's K loop is cut
 // into equal parts of at most Lmax stages, Lmax the shortest for which there are at most w units per
-// SM; w is the one with the least w Lmax, plus kTcOver where that cuts any tile (the stages that the
-// trip through the workspace costs, about 6 us). Longest first, dealt to the CTAs in turn.
+// SM; w is the one with the least w Lmax, plus kTcOver where that cuts any tile (the trip through
+// the workspace, in stages; 6 to 18 give the same times). Longest first, dealt to the CTAs in turn.
 constexpr int kTcOver = 12, kTcMaxParts = 16;
 static std::vector<TcUnit> tc_units(const std::vector<TcObj>& objs, int mats, int nsm, int* slots) {
   struct T { int obj, row0, mat, nk; };
