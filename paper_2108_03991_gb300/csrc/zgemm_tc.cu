@@ -17,21 +17,25 @@
 // or slice lose bits: 5 exponent bits. A column of Z falls by 2^-100 along a bar of 30 skin depths, and
 // a unit vector's product has to return it.) Two TF32 parts take as many MMAs and more shared memory.
 //
-// Layout. B is packed once per call from x into [3 parts][N][K_tot]: every object's K range starts at a
-// multiple of 32 values, and 32 values of a row are 64 bytes (zeros past the object's 2 n values). A is
-// read in place through one 2-D tensor map per object (inner extent 2n floats, rows n, row pitch 8 ld
-// bytes): TMA fills the K tail and the rows past n with zeros; the landed FP32 tile is turned in place
-// into rows of 32 first parts and 32 second parts, its third parts go to a tile beside it. Shared-memory
-// tiles are K-major; rows of 128 bytes (A) have the 128-byte swizzle, rows of 64 bytes (A3, B) the
-// 64-byte one. The parts of B follow each other, so that one MMA multiplies A1 by two or three of them.
+// Layout. B is packed once per call from x, stage by stage as shared memory holds it: [stage][3
+// parts][NP rows][64 bytes, swizzled], every object's stages (32 values each, zeros past the object's 2 n)
+// one after another, so that a stage is one contiguous bulk copy. (Rows of all objects' K values behind a
+// tensor map put a stage's rows megabytes apart: C of 1,024 rings with 64 right-hand sides took
+// 5.3 ms instead of 2.25.) A is read in place through one 2-D tensor map per object (inner extent 2n floats,
+// rows n, row pitch 8 ld bytes): TMA fills the K tail and the rows past n with zeros; the landed FP32
+// tile is turned in place into rows of 32 first parts and 32 second parts, its third parts go to a tile
+// beside it. Shared-memory tiles are K-major; rows of 128 bytes (A) have the 128-byte swizzle, rows of 64
+// bytes (A3, B) the 64-byte one. The parts of B follow each other, so that one MMA multiplies A1 by two
+// or three of them.
 //
 // A product is bound by shared memory (a stage of 32 K values moves 168 KB through it at N = 128: the
 // landing tiles, the conversion, the operands of 10 MMAs) and by the HBM reads of the blocks, so both
 // matrices go in one launch of persistent CTAs and the K loops of the tiles are cut into units that
 // load them evenly (tc_units). Z and C together, packing included (us, 64 right-hand sides): six bars of
-// 240-1,920 edges 79, one bar of 2,016 46, 16 rings of 912 91 (257, 263, 144 with one launch per matrix
-// and a CTA per tile in TF32; 69, 40, 72 with two FP16 parts); 16 right-hand sides 61, 36, 68; 128 of
-// them 121, 64, 132 (539, 446, 262; 100, 56, 105); 144 rings 414 at 1 (HBM-bound), 637 at 64 (395, 468).
+// 240-1,920 edges 78, one bar of 2,016 45, 16 rings of 912 90 (257, 263, 144 with one launch per matrix
+// and a CTA per tile in TF32; 69, 40, 72 with two FP16 parts); 16 right-hand sides 58, 33, 66; 128 of
+// them 120, 63, 128 (539, 446, 262; 100, 56, 105). C alone of 576 rings 815 at 16 (HBM-bound), 1,299 at
+// 64, 2,153 at 128 (786, 1,130, 2,242 with two FP16 parts behind a tensor map).
 // Error against 64 bits on the bars 4.5e-7, on the rings 2.2e-6 (TF32 6.6e-6), the accumulator's.
 // Every wait is bounded: on a timeout the CTA records an error (err[0], kept across products)
 // and raises the launch's abort flag (err[1], cleared before each launch), waits (with a short
@@ -71,7 +75,7 @@ struct TcUnit {  // stages [k0, k1) of one 128-row tile of one block of Z (mat 0
 };
 struct TcObj {   // per object: size, first unknown, first K column in the packed B
   int32_t n, xoff;
-  int64_t koff;
+  int64_t koff;  // first stage in the packed B
 };
 
 // K-major operand in shared memory with the 128-byte swizzle: rows of 128 bytes, 8-row groups
@@ -179,20 +183,21 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, const in
   return false;
 }
 
-// B from x: rows 2r and 2r + 1 of right-hand side r < R (zero rows up to NP) of the three parts (pstride
-// words apart), one CTA per object and right-hand side: the slice's 2 n values, zeros up to the object's
-// padded length; a word holds two values
+// B from x: rows 2r and 2r + 1 of right-hand side r < R (zero rows up to NP) of the three parts, one CTA
+// per object and right-hand side: the slice's 2 n values, zeros up to the object's last stage. A word
+// holds two values, 16 words are a row's part of a stage; the two rows of r share a 128-byte line
 __global__ void __launch_bounds__(256) k_tc_pack(const float2* __restrict__ x, int64_t vstride, int R,
-                                                 const TcObj* __restrict__ objs, int64_t ktot,
-                                                 uint32_t* __restrict__ b, int64_t pstride) {
+                                                 const TcObj* __restrict__ objs, int NP,
+                                                 uint32_t* __restrict__ b) {
   const TcObj o = objs[blockIdx.x];
   const int r = blockIdx.y;
   const float2* xs = x + r * vstride + o.xoff;
-  uint32_t* p = b + 2 * r * ktot + o.koff;
+  uint32_t* p0 = b + (o.koff * 3 * NP + 2 * r) * 16;
   for (int k = threadIdx.x; k < (o.n + 15 & ~15); k += 256) {
     const float2 v = r < R && k < o.n ? xs[k] : make_float2(0.f, 0.f);
-    tc_split(v.x, -v.y, p + k, p + pstride + k, p + 2 * pstride + k);
-    tc_split(v.y, v.x, p + ktot + k, p + pstride + ktot + k, p + 2 * pstride + ktot + k);
+    uint32_t* p = p0 + (int64_t)(k >> 4) * (48 * NP) + (((k >> 2 & 3) ^ (r & 3)) * 4 + (k & 3));
+    tc_split(v.x, -v.y, p, p + 16 * NP, p + 32 * NP);
+    tc_split(v.y, v.x, p + 16, p + 16 * NP + 16, p + 32 * NP + 16);
   }
 }
 
@@ -241,7 +246,7 @@ __device__ __forceinline__ void tc_convert_row(uint8_t* tile, int row) {
 // unit that finishes last, four warps on one SM, took 50 us for it).
 template <int NP>
 __global__ void __launch_bounds__(tc_threads<NP>(), 1)
-    k_zgemm_tc(const __grid_constant__ CUtensorMap mb, const CUtensorMap* __restrict__ mz,
+    k_zgemm_tc(const uint32_t* __restrict__ b, const CUtensorMap* __restrict__ mz,
                const CUtensorMap* __restrict__ mc, const TcUnit* __restrict__ units, int nunit,
                const int32_t* __restrict__ nst, const TcObj* __restrict__ objs,
                float2* __restrict__ yz, float2* __restrict__ yc, int64_t vstride, int R,
@@ -357,11 +362,9 @@ __global__ void __launch_bounds__(tc_threads<NP>(), 1)
             break;
           }
           uint8_t* st = base + slot * L::kStage;
-          const int kx = (int)(o.koff + (int64_t)kc * (kTcK / 2));  // in words of two values
           mbar_arrive_tx(&full[slot], L::kTx);
           tma_load_2d(st, mA, kc * kTcK, u.row0, &full[slot]);
-#pragma unroll
-          for (int p = 0; p < 3; ++p) tma_load_2d(st + L::kB + p * L::kBp, &mb, kx, p * NP, &full[slot]);
+          bulk_g2s(st + L::kB, b + (o.koff + kc) * (48 * NP), 3 * L::kBp, &full[slot]);
           ++issued;
           if (++slot == S) {
             slot = 0;
@@ -507,8 +510,8 @@ struct TcState {
     int n = 0, ncut = 0, slots = 0, ctas = 0;
   } units[3];                 // Z alone, C alone, both
   TcObj* objs = nullptr;
-  int64_t ktot = 0;           // 32-bit words per row of the packed B
-  uint32_t* b = nullptr;      // packed B, [3][NP][ktot]
+  int64_t ktot = 0;           // stages of the packed B
+  uint32_t* b = nullptr;      // packed B, [ktot][3][NP][16]
   float4* part = nullptr;     // partial sums of tiles cut along K
   int np_cap = 0;
   int* err = nullptr;         // [2]: a wait timed out in some product (sticky); this launch gave up
@@ -535,21 +538,20 @@ static TcEncode tc_encoder() {
   return fn;
 }
 
-// 2-D tensor map of 4-byte elements, inner extent `inner` of them, `rows` rows `pitch` bytes apart, box
-// of box_cols (32 or 16: 128 or 64 bytes, swizzled over that width) x box_rows, zero fill outside
+// 2-D FP32 tensor map, inner extent `inner` floats, `rows` rows `pitch` bytes apart, box of
+// 32 floats x box_rows, 128-byte swizzle, zero fill outside
 static int tc_map(TcEncode enc, CUtensorMap* m, const void* base, int64_t inner, int64_t rows,
-                  int64_t pitch, int box_cols, int box_rows) {
+                  int64_t pitch, int box_rows) {
   const cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)pitch};
-  const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+  const cuuint32_t box[2] = {(cuuint32_t)kTcK, (cuuint32_t)box_rows};
   const cuuint32_t es[2] = {1, 1};
   if ((reinterpret_cast<uintptr_t>(base) & 15) || (pitch & 15)) {
     set_error("tensor-core product: operand not 16-byte aligned");
     return BEM_EINVAL;
   }
   const CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides,
-                         box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                         box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                         box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_error("tensor-core product: cuTensorMapEncodeTiled failed (%d)", (int)r);
@@ -633,14 +635,10 @@ static int tc_prepare(aim_ctx* c, TcState** out) {
   for (int i = 0, xo = 0; i < c->nobj && rc == BEM_OK; ++i) {
     const int n = c->e1[i] - c->e0[i], ld = c->zld[i];
     objs[i] = TcObj{n, xo, ktot};
-    ktot += round_up(n, 16);
-    rc = tc_map(enc, &mz[i], c->f32.Z + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcK, kTcM);
-    if (rc == BEM_OK) rc = tc_map(enc, &mc[i], c->f32.C + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcK, kTcM);
+    ktot += round_up(n, 16) / 16;
+    rc = tc_map(enc, &mz[i], c->f32.Z + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcM);
+    if (rc == BEM_OK) rc = tc_map(enc, &mc[i], c->f32.C + c->zoff[i], 2 * (int64_t)n, n, 8 * (int64_t)ld, kTcM);
     xo += n;
-  }
-  if (rc == BEM_OK && ktot > INT32_MAX) {
-    set_error("tensor-core product: more than 2^31 unknowns");
-    rc = BEM_EINVAL;
   }
   t->ktot = ktot;
   auto up = [&](void** p, const void* h, size_t bytes) {
@@ -683,15 +681,14 @@ static int tc_prepare(aim_ctx* c, TcState** out) {
 }
 
 template <int NP>
-static int tc_launch(TcState* t, const CUtensorMap& mb, float2* yz, float2* yc, int64_t vstride, int R,
-                     cudaStream_t s) {
+static int tc_launch(TcState* t, float2* yz, float2* yc, int64_t vstride, int R, cudaStream_t s) {
   constexpr uint32_t kSmem = TcSmem<NP>::kBytes;
   static_assert(kSmem <= 227 * 1024, "shared memory per CTA");
   const TcState::Units& q = t->units[yz && yc ? 2 : yz ? 0 : 1];
   // per call: the attribute belongs to the current device (cheap next to the product)
   BEM_CUDA(cudaFuncSetAttribute(k_zgemm_tc<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
   BEM_CUDA(cudaMemsetAsync(t->err + 1, 0, sizeof(int), s));
-  k_zgemm_tc<NP><<<q.ctas, tc_threads<NP>(), kSmem, s>>>(mb, t->mz, t->mc, q.d, q.n, q.nst, t->objs, yz, yc,
+  k_zgemm_tc<NP><<<q.ctas, tc_threads<NP>(), kSmem, s>>>(t->b, t->mz, t->mc, q.d, q.n, q.nst, t->objs, yz, yc,
                                                          vstride, R, t->part, t->err);
   if (q.ncut > 0)
     k_tc_reduce<NP><<<dim3(q.ncut, (2 * R + 15) / 16), kTcM, 0, s>>>(q.cut, t->objs, t->part, yz, yc, vstride, R);
@@ -704,7 +701,6 @@ int internal_tc(aim_ctx* c, const float2* h, float2* e, float2* heq, int nrhs, c
   TcState* t = nullptr;
   BEM_TRY(tc_prepare(c, &t));
   if (t->units[0].n == 0) return BEM_OK;
-  TcEncode enc = tc_encoder();
   const int64_t ne = c->ne;
   for (int r0 = 0; r0 < nrhs; r0 += kTcMaxRhs) {
     const int R = std::min(kTcMaxRhs, nrhs - r0);
@@ -716,7 +712,7 @@ int internal_tc(aim_ctx* c, const float2* h, float2* e, float2* heq, int nrhs, c
       t->b = nullptr;
       t->part = nullptr;
       t->np_cap = 0;
-      const size_t bytes = (size_t)3 * NP * t->ktot * sizeof(uint32_t);
+      const size_t bytes = (size_t)3 * NP * 16 * t->ktot * sizeof(uint32_t);
       int slots = 0;
       for (const TcState::Units& q : t->units) slots = std::max(slots, q.slots);
       const size_t pbytes = (size_t)slots * kTcM * NP * sizeof(float) + 16;
@@ -726,13 +722,11 @@ int internal_tc(aim_ctx* c, const float2* h, float2* e, float2* heq, int nrhs, c
       }
       t->np_cap = NP;
     }
-    CUtensorMap mb;  // 16 words of a row are one stage
-    BEM_TRY(tc_map(enc, &mb, t->b, t->ktot, 3 * NP, 4 * t->ktot, kTcK / 2, NP));
-    k_tc_pack<<<dim3(c->nobj, NP / 2), 256, 0, s>>>(h + r0 * ne, ne, R, t->objs, t->ktot, t->b, NP * t->ktot);
+    k_tc_pack<<<dim3(c->nobj, NP / 2), 256, 0, s>>>(h + r0 * ne, ne, R, t->objs, NP, t->b);
     BEM_CUDA(cudaGetLastError());
     float2* yz = e ? e + r0 * ne : nullptr;
     float2* yc = heq ? heq + r0 * ne : nullptr;
-#define BEM_TC(NPV) BEM_TRY(tc_launch<NPV>(t, mb, yz, yc, ne, R, s))
+#define BEM_TC(NPV) BEM_TRY(tc_launch<NPV>(t, yz, yc, ne, R, s))
     switch (NP) {
       case 32: BEM_TC(32); break;
       case 64: BEM_TC(64); break;
